@@ -287,13 +287,14 @@ int sr_plan(int64_t n, int dtype, const sr_config* cfg, sr_config* resolved);
  * grid whatever the segment lengths; segments crossing a warp boundary are
  * finished by the configured grid stage: SR_TWO_KERNEL, SR_GRID_SYNC,
  * SR_LAST_BLOCK (per-segment tickets; the SR_AUTO default for floating-point
- * inputs) or SR_ATOMIC (out zeroed first; FP order not deterministic; the
- * SR_AUTO default for SR_I32, whose int64 sums are exact in any order).  All
- * other forms are deterministic.
+ * inputs and from 2^19 segments) or SR_ATOMIC (out zeroed first; FP order not
+ * deterministic; the SR_AUTO default for SR_I32 below 2^19 segments, whose
+ * int64 sums are exact in any order).  All other forms are deterministic.
  * Load path: rows of 16/32-byte vectors loaded into registers (LDG), or with
  * SR_F_BULK each warp streams its piece through its own ring of `stages`
  * (2..8, default 2) chunks of `unroll` rows (2, 4 or 8; default 4) in shared
- * memory, one cp.async.bulk per chunk (the TMA form; every wait bounded, an
+ * memory, one cp.async.bulk per chunk (the TMA form, which resolves segment
+ * ends once per chunk and so also suits short segments; every wait bounded, an
  * expired one reported as SR_ERR_TIMEOUT by sr_stream_status).  Without an
  * explicit shape (vec_bytes, unroll, block_threads and stages all 0) calls
  * with 32768 or more segments take the TMA form, fewer the LDG one.

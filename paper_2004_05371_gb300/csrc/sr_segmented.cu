@@ -33,6 +33,10 @@ constexpr int kKnownSegFlags =
 // the load-path / form flags, at most one of which a segmented call may set
 constexpr int kSegFormFlags =
     SR_F_DENSE_SEGMENTS | SR_F_BULK | SR_F_WARP_SEGMENTS | SR_F_LANE_SEGMENTS | SR_F_ADAPTIVE_SEGMENTS;
+// int32, no stage given: segments up to which the output is zeroed and added to
+// atomically.  2^21 segments of 16: 61.8 us with the 16 MiB zeroed, 54.6 with
+// tickets; 90,000 of 16: 9.6 against 11.7.
+constexpr int64_t kSegZeroMax = 1 << 19;
 constexpr int64_t kSegBulkMin = 32768;  // segments from which the default shape is the TMA form
 
 const void* seg_adapt_kernel(int dtype, bool comp, int vec, int unroll) {
@@ -114,8 +118,9 @@ int seg_plan(int64_t nseg, int dtype, const sr_config& c, const DeviceInfo& d, S
     p.stage = c.variant & SR_STAGE_MASK;
     // SR_AUTO: last-block-done; for int32 the atomic finish (int64 sums are
     // exact in any order, so it stays deterministic, and it is 2-3 % faster:
-    // no ticket, no second read of the carries)
-    if (p.stage == SR_AUTO) p.stage = dtype == SR_I32 ? SR_ATOMIC : SR_LAST_BLOCK;
+    // no ticket, no second read of the carries), until the zeroing of 8 bytes
+    // per segment costs more than the tickets do (kSegZeroMax segments)
+    if (p.stage == SR_AUTO) p.stage = dtype == SR_I32 && nseg < kSegZeroMax ? SR_ATOMIC : SR_LAST_BLOCK;
     // defaults from autotuner sweeps of 10,000 lognormal segments (~2^28 FP32):
     // 32-byte vectors, 8 rows in flight per warp, 256-thread CTAs
     p.vec = c.vec_bytes ? c.vec_bytes : 32;
@@ -164,14 +169,15 @@ int seg_plan(int64_t nseg, int dtype, const sr_config& c, const DeviceInfo& d, S
         if (!c.block_threads) p.block = 512;
     }
     // Without an explicit shape, many segments (kSegBulkMin or more) take the TMA
-    // form: measured 1.02-1.41x the LDG default from 100,000 to 16M segments of
-    // ~2^28 elements, 1 % behind it at 10,000.
+    // form, which resolves segment ends once per chunk: from 100,000 to 16M
+    // segments of ~2^28 elements it takes 164-229 us, the LDG default 192-3361; at
+    // 10,000 it is 1-3 % behind.
     const bool shape_given = c.vec_bytes || c.unroll || c.block_threads || c.stages;
     p.bulk = (c.variant & SR_F_BULK) != 0 || (!shape_given && !p.dense && !p.warp && !p.lane && nseg >= kSegBulkMin);
-    if (p.bulk) {  // per-warp ring: stages x (unroll rows of 32 vectors) + one mbarrier per stage
+    if (p.bulk) {  // per warp: stages x (unroll rows of 32 vectors + one mbarrier), and the strip table
         if (!c.unroll) p.unroll = 4;
         p.stages = c.stages ? c.stages : 2;
-        p.smem = (size_t)(p.block / 32) * p.stages * ((size_t)p.unroll * 32 * p.vec + 8);
+        p.smem = (size_t)(p.block / 32) * (p.stages * ((size_t)p.unroll * 32 * p.vec + 8) + kStripTableBytes);
         if (p.smem > (size_t)d.smem_per_block_optin) return SR_ERR_LAUNCH;
     }
     if (!seg_kernels(dtype, p.comp, p.vec, p.unroll, p.dense, p.bulk, p.warp, p.lane, &p.main, &p.fin))

@@ -1,7 +1,7 @@
 // Segmented (batched) sum: out[s] = sum of x[offsets[s] .. offsets[s+1]).
 // Kernel templates, instantiated per input dtype by sr_segmented_<dtype>.cu.
 //
-// Work split: the concatenated range [offsets[0], offsets[nseg]) is cut into
+// Work split of the flat forms: the concatenated range [offsets[0], offsets[nseg]) is cut into
 // W equal, vector-aligned pieces of E elements, one per warp of the grid, so
 // the load is balanced whatever the segment lengths.  Segment s is *owned*
 // by the warp whose piece contains offsets[s].  Each warp
@@ -66,6 +66,44 @@ __device__ __forceinline__ int64_t warp_lower_bound(const int64_t* off, int64_t 
     int64_t lo = 0, hi = nseg;  // answer in [lo, hi]
     while (hi - lo > 32) lb_round(off, key, lane, lo, hi);
     return lb_final(off, key, lane, lo, hi);
+}
+
+// The first s in [0, nseg] with offsets[s] >= key, and the offsets around it.
+// On return lane k holds offsets[wb + k] in `win` (INT64_MAX past offsets[nseg])
+// and the answer r lies in [wb, wb + 30], so offsets[r] and offsets[r + 1] are
+// in the window.  The first probe spreads the lanes at power-of-two distances
+// around `guess`, the answer for equal segments: for layouts near it that is
+// one round of loads instead of log32(nseg) (whole warp calls).
+__device__ __forceinline__ int64_t warp_search(const int64_t* off, int64_t nseg, int64_t key, int64_t guess, int lane,
+                                               int64_t& wb, int64_t& win) {
+    int64_t lo = 0, hi = nseg;  // the answer is in [lo, hi]
+    if (nseg > 30) {
+        const int64_t i = lane < 16 ? guess - (1 << (15 - lane)) : guess + (1 << (lane - 16)) - 1;
+        const bool pred = i >= nseg || (i >= 0 && __ldg(off + i) >= key);
+        const unsigned m = __ballot_sync(0xffffffffu, pred);
+        const int k = m ? __ffs(m) - 1 : 32;
+        const int64_t below = __shfl_sync(0xffffffffu, i, k > 0 ? k - 1 : 0);
+        const int64_t at = __shfl_sync(0xffffffffu, i, k < 32 ? k : 31);
+        if (k > 0 && below >= 0) lo = below + 1;
+        if (k < 32 && at < nseg) hi = at;
+    }
+    while (hi - lo > 30) {
+        const int64_t step = (hi - lo + 31) / 32;
+        const int64_t i = lo + (int64_t)lane * step;
+        const bool pred = (i < hi) ? (__ldg(off + i) >= key) : true;
+        const unsigned m = __ballot_sync(0xffffffffu, pred);
+        if (m == 0) {
+            lo = lo + 31 * step + 1;
+        } else {
+            const int k = __ffs(m) - 1;
+            const int64_t ik = lo + (int64_t)k * step;
+            hi = ik < hi ? ik : hi;
+            if (k > 0) lo = lo + (int64_t)(k - 1) * step + 1;
+        }
+    }
+    wb = lo;
+    win = (lo + lane <= nseg) ? __ldg(off + lo + lane) : INT64_MAX;
+    return lo + __ffs(__ballot_sync(0xffffffffu, lo + lane >= hi || win >= key)) - 1;
 }
 
 // Element j of a vector held as 32-bit words (the masked slow path; j is a
@@ -205,12 +243,7 @@ template <class A> __device__ __forceinline__ void span_arrive(const SegParams& 
 // boundary.
 constexpr int kScanMin = 3;  // boundaries in a row from which the warp-wide pass pays
 
-// BULK: the warp's vector body streams through its own ring of p.stages
-// chunks of UNROLL rows in shared memory, one cp.async.bulk per chunk issued by
-// lane 0 and completing on the chunk stage's mbarrier (every wait bounded by
-// p.limit_ns; on expiry the warp records SR_ERR_TIMEOUT, waits for the copies
-// it issued, and stops).  No registers hold rows in flight.
-template <int DT, bool COMP, int VB, int UNROLL, bool DENSE, bool BULK>
+template <int DT, bool COMP, int VB, int UNROLL, bool DENSE>
 __global__ void __launch_bounds__(512, 1) seg_kernel(const SegParams p) {
     using A = typename Acc<DT, COMP>::T;
     constexpr int EB = SegElem<DT>::v;
@@ -242,36 +275,11 @@ __global__ void __launch_bounds__(512, 1) seg_kernel(const SegParams p) {
     const unsigned char* body = p.x + a0 * EB;
 
     // first batch of rows in flight before the segment search
-    uint32_t buf[BULK ? 1 : UNROLL][W];
-    constexpr uint32_t CHUNK = (uint32_t)UNROLL * 32u * VB;  // bytes of one ring stage
-    const int64_t nchunks = (nrows + UNROLL - 1) / UNROLL;
-    uint32_t ring = 0, bars = 0;
-    // lane 0: copy chunk k of the body into its ring stage
-    auto issue = [&](int64_t k) {
-        const int64_t v0 = k * (UNROLL * 32);
-        if (v0 >= nvec) return;
-        const int64_t nv = (nvec - v0 < UNROLL * 32) ? nvec - v0 : (int64_t)UNROLL * 32;
-        const int st = (int)(k % p.stages);
-        mbar_arrive_expect_tx(bars + 8u * st, (uint32_t)(nv * VB));
-        bulk_g2s(ring + (uint32_t)st * CHUNK, body + v0 * VB, (uint32_t)(nv * VB), bars + 8u * st);
-    };
-    if constexpr (BULK) {
-        extern __shared__ __align__(128) unsigned char seg_dsm[];
-        const int wib = threadIdx.x >> 5, nwib = blockDim.x >> 5;
-        ring = smem_u32(seg_dsm) + (uint32_t)(wib * p.stages) * CHUNK;
-        bars = smem_u32(seg_dsm) + (uint32_t)(nwib * p.stages) * CHUNK + (uint32_t)(wib * p.stages) * 8u;
-        if (lane == 0) {
-            for (int st = 0; st < p.stages; ++st) mbar_init(bars + 8u * st, 1);
-            mbar_fence_init();
-            for (int64_t k = 0; k < p.stages && k < nchunks; ++k) issue(k);
-        }
-        __syncwarp();
-    } else {
+    uint32_t buf[UNROLL][W];
 #pragma unroll
-        for (int u = 0; u < UNROLL; ++u) {
-            const int64_t v = (int64_t)u * 32 + lane;
-            if (v < nvec) ldg_vec(body + v * VB, buf[u]);
-        }
+    for (int u = 0; u < UNROLL; ++u) {
+        const int64_t v = (int64_t)u * 32 + lane;
+        if (v < nvec) ldg_vec(body + v * VB, buf[u]);
     }
 
     const int64_t s_begin = warp_lower_bound(p.offsets, p.nseg, base + w * E, lane);
@@ -462,66 +470,577 @@ __global__ void __launch_bounds__(512, 1) seg_kernel(const SegParams p) {
     };
 
     scalar_chunk(lo, a0);
-    bool bail = false;
-    if constexpr (BULK) {
-        for (int64_t k = 0; k < nchunks; ++k) {
-            const int st = (int)(k % p.stages);
-            const uint32_t par = (uint32_t)((k / p.stages) & 1);
-            if (!__all_sync(0xffffffffu, mbar_wait_bounded(bars + 8u * st, par, p.limit_ns))) {
-                if (lane == 0) {
-                    atomicOr(p.err, kErrTimeout);
-                    // leave no copy writing this CTA's shared memory: wait for the ones
-                    // issued (chunks k .. k + stages - 1), bounded separately (>= 1 s)
-                    const uint64_t drain = p.limit_ns > 1000000000ull ? p.limit_ns : 1000000000ull;
-                    for (int64_t j = k; j < nchunks && j < k + p.stages; ++j)
-                        mbar_wait_bounded(bars + 8u * (uint32_t)(j % p.stages), (uint32_t)((j / p.stages) & 1), drain);
-                }
-                bail = true;
-                break;
-            }
-            const uint32_t sb = ring + (uint32_t)st * CHUNK + (uint32_t)lane * VB;
+    for (int64_t r = 0; r < nrows; r += UNROLL) {
+        if (r > 0) {
 #pragma unroll
             for (int u = 0; u < UNROLL; ++u) {
-                const int64_t r = k * UNROLL + u;
-                if (r < nrows) {
-                    uint32_t words[W];
-#pragma unroll
-                    for (int h = 0; h < W / 4; ++h) {
-                        uint32_t t4[4];
-                        lds_vec(sb + (uint32_t)u * 32u * VB + 16u * h, t4);
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) words[4 * h + i] = t4[i];
-                    }
-                    row(r, words);
-                }
-            }
-            __syncwarp();  // every lane has read the stage
-            if (lane == 0) {
-                fence_proxy_async_smem();
-                issue(k + p.stages);
+                const int64_t v = (r + u) * 32 + lane;
+                if (v < nvec) ldg_vec(body + v * VB, buf[u]);
             }
         }
-    } else {
-        for (int64_t r = 0; r < nrows; r += UNROLL) {
-            if (r > 0) {
 #pragma unroll
-                for (int u = 0; u < UNROLL; ++u) {
-                    const int64_t v = (r + u) * 32 + lane;
-                    if (v < nvec) ldg_vec(body + v * VB, buf[u]);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < UNROLL; ++u)
-                if (r + u < nrows) row(r + u, buf[u]);
+        for (int u = 0; u < UNROLL; ++u)
+            if (r + u < nrows) row(r + u, buf[u]);
+    }
+    scalar_chunk(hi_al, hi);
+    // the segment holding the piece's last element, then any (empty) segment
+    // this warp owns that starts at or after hi
+    while (cur < p.nseg && cur_start < next_lo) emit_advance();
+
+    if (p.stage == kStageTwoKernel || p.stage == kStageGridSync) {
+        if (lane == 0) p.last_seg[w] = spanning;
+    }
+    if (p.stage == kStageGridSync) {
+        cg::grid_group g = cg::this_grid();
+        if (!g.is_valid()) {
+            if (threadIdx.x == 0) atomicOr(p.err, 2);
+            return;
+        }
+        g.sync();
+        if (spanning >= 0) {
+            const int64_t end = __ldg(p.offsets + spanning + 1);
+            finish_span<A>(p, spanning, w, (end - 1 - base) / E, lane);
         }
     }
-    if (!bail) {
-        scalar_chunk(hi_al, hi);
+}
+
+// ------------------------------------------------------- TMA form (strips)
+// SR_F_BULK: the flat split with each warp's vector body streamed through its
+// own ring of p.stages chunks of UNROLL rows of 32 vectors in shared memory,
+// one cp.async.bulk per chunk issued by lane 0 and completing on the chunk
+// stage's mbarrier (every wait bounded by p.limit_ns; on expiry the warp records
+// SR_ERR_TIMEOUT, waits for the copies it issued, and stops).
+//
+// A chunk is cut into 32 strips, one per lane: strip t is its t-th run of
+// UNROLL * VB contiguous bytes, NV 16-byte vectors.  Segment ends are resolved
+// once per chunk instead of once per row or per segment:
+//   - a segment inside one strip is summed by the lane that holds its end in
+//     the offsets window, straight from shared memory;
+//   - every lane sums its strip's vectors before the strip's first boundary
+//     (head) and from its last one on (tail), the two boundary vectors split
+//     element by element; one segmented scan over the lanes then closes every
+//     segment that crosses a strip, and its last value is the segment open at
+//     the chunk's end.
+// Where every segment of a chunk is short, the strips are left out: each is
+// summed by its own lane (OwnBytes, below).
+//
+// Resolving the ends row by row, with a warp reduction for each (as the LDG
+// kernel does), bounded the ring by its instructions: it read 1M segments of 268
+// BF16 values at 1.8 TB/s.  Now a chunk with ends in it costs about 450 warp
+// instructions whatever their number, where HBM leaves time for some 650.
+// Device time before and now (~2^28 elements unless said otherwise):
+//   f32   1M x 268             343 -> 178 us      f32  4M lognormal    1013 -> 200 us
+//   f32   4M x 64              915 -> 189         f32  16M x 16        3110 -> 229
+//   bf16  1M x 268 (0..536)    297 -> 102         fp8  100k lognormal   160 ->  63
+//   i32   2^21 x 16 (0..32)    525 ->  55         bf16 4M x 39, lognormal 868 -> 115
+// What bounds it now: instructions (55-70 % of the issue slots) from about five
+// ends per chunk up, HBM below.  80 registers, so three 256-thread CTAs (24 warps)
+// are resident with two 4 KiB stages each: 16 warps of 112 registers took 4 %
+// less on long segments and 8-12 % more on short ones.
+
+// Sum of the elements in one 16-byte vector (four 32-bit words).
+template <int DT, class A> __device__ __forceinline__ A vec_total(const uint32_t (&r)[4]) {
+    if constexpr (DT == kDtI32) {
+        long long s = (long long)(int)r[0];
+#pragma unroll
+        for (int w = 1; w < 4; ++w) asm("mad.wide.s32 %0, %1, 1, %0;" : "+l"(s) : "r"(r[w]));
+        return s;
+    } else if constexpr (DT == kDtFP8) {
+        const float v = AccVec<kDtFP8, float, 4>::vec_sum(r);  // 16 values: exact
+        if constexpr (std::is_same<A, Pair>::value) return Pair{v, 0.f};
+        else return v;
+    } else if constexpr (std::is_same<A, Pair>::value) {
+        Pair t[4];
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            if constexpr (DT == kDtF32) t[w] = Pair{__uint_as_float(r[w]), 0.f};
+            else two_sum(__uint_as_float(r[w] << 16), __uint_as_float(r[w] & 0xffff0000u), t[w].s, t[w].c);
+        }
+        return Op<Pair>::add(Op<Pair>::add(t[0], t[1]), Op<Pair>::add(t[2], t[3]));
+    } else if constexpr (DT == kDtBF16) {
+        const float a = bf16_hi_add(r[1], bf16_lo_add(r[1], bf16_hi_add(r[0], __uint_as_float(r[0] << 16))));
+        const float b = bf16_hi_add(r[3], bf16_lo_add(r[3], bf16_hi_add(r[2], __uint_as_float(r[2] << 16))));
+        return __fadd_rn(a, b);
+    } else {
+        return __fadd_rn(__fadd_rn(__uint_as_float(r[0]), __uint_as_float(r[1])),
+                         __fadd_rn(__uint_as_float(r[2]), __uint_as_float(r[3])));
+    }
+}
+
+// A running sum of whole vectors: the accumulator type itself, or for plain
+// binary32 two partial sums in one packed register pair (PTX add.rn.f32x2:
+// each half rounds like the scalar add, in half the instructions).
+template <int DT, class A> struct VecPart {
+    A v;
+    __device__ __forceinline__ static VecPart zero() { return VecPart{Op<A>::zero()}; }
+    __device__ __forceinline__ static VecPart of(const uint32_t (&r)[4]) { return VecPart{vec_total<DT, A>(r)}; }
+    __device__ __forceinline__ void add(const VecPart& b) { v = Op<A>::add(v, b.v); }
+    __device__ __forceinline__ A total() const { return v; }
+};
+template <> struct VecPart<kDtF32, float> {
+    float x, y;
+    __device__ __forceinline__ static VecPart zero() { return VecPart{0.f, 0.f}; }
+    __device__ __forceinline__ static VecPart sum(float ax, float ay, float bx, float by) {
+        VecPart t;
+        asm("{ .reg .b64 a, b, c;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n"
+            " add.rn.f32x2 c, a, b;\n mov.b64 {%0, %1}, c; }"
+            : "=f"(t.x), "=f"(t.y)
+            : "f"(ax), "f"(ay), "f"(bx), "f"(by));
+        return t;
+    }
+    __device__ __forceinline__ static VecPart of(const uint32_t (&r)[4]) {
+        return sum(__uint_as_float(r[0]), __uint_as_float(r[1]), __uint_as_float(r[2]), __uint_as_float(r[3]));
+    }
+    __device__ __forceinline__ void add(const VecPart& b) { *this = sum(x, y, b.x, b.y); }
+    __device__ __forceinline__ float total() const { return __fadd_rn(x, y); }
+};
+
+// The low n bits (n <= 0: none, n >= 32: all).
+__device__ __forceinline__ uint32_t low_bits(int n) {
+    uint32_t above;  // PTX shl: 0 from 32 on
+    asm("shl.b32 %0, %1, %2;" : "=r"(above) : "r"(0xffffffffu), "r"(max(n, 0)));
+    return ~above;
+}
+// Zero the elements of a vector at or after index n (keep_below) or before it
+// (keep_from); 0 <= n <= 16 / EB.  A zeroed word is +0 in every input type.
+template <int EB> __device__ __forceinline__ void keep_below(uint32_t (&r)[4], int n) {
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+        if constexpr (EB == 4) r[w] = w < n ? r[w] : 0u;
+        else r[w] &= low_bits(8 * EB * n - 32 * w);
+    }
+}
+template <int EB> __device__ __forceinline__ void keep_from(uint32_t (&r)[4], int n) {
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+        if constexpr (EB == 4) r[w] = w >= n ? r[w] : 0u;
+        else r[w] &= ~low_bits(8 * EB * n - 32 * w);
+    }
+}
+
+constexpr int kAheadOffsets = 256;   // offsets fetched into L2 this far ahead of the window
+// Longest segment (bytes) one lane sums alone, about where that costs a chunk
+// as many instructions as the strips do.
+template <int DT> struct OwnBytes { static constexpr int v = 256; };
+template <> struct OwnBytes<kDtI32> { static constexpr int v = 192; };
+template <> struct OwnBytes<kDtBF16> { static constexpr int v = 192; };
+template <> struct OwnBytes<kDtFP8> { static constexpr int v = 128; };
+
+template <int DT, bool COMP, int VB, int UNROLL>
+__global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
+    using A = typename Acc<DT, COMP>::T;
+    using VP = VecPart<DT, A>;
+    constexpr int EB = SegElem<DT>::v;
+    constexpr int PV = VB / EB;                             // elements per vector of the flat split
+    constexpr uint32_t CHUNK = (uint32_t)UNROLL * 32u * VB;  // bytes of one ring stage
+    constexpr int CE = (int)CHUNK / EB;                     // elements of a chunk
+    constexpr int SE = CE / 32;                             // elements of a strip (a power of two)
+    constexpr int EV = 16 / EB;                             // elements of a 16-byte vector
+    constexpr int NV = SE / EV;                             // 16-byte vectors of a strip
+    constexpr int kOwn = OwnBytes<DT>::v / EB;
+    // FP8 and compensated BF16 vectors take 40 to 50 instructions each: with their
+    // loops unrolled the warps wait for instructions (FP8: 72 us against 63 on
+    // 100,000 lognormal segments of 2^28 elements)
+    constexpr bool kCompact = DT == kDtFP8 || (COMP && DT == kDtBF16);
+    constexpr int UN = kCompact && NV > 2 ? 2 : NV;
+    grid_dependency_wait();
+    allow_dependents();
+    if (p.bad != nullptr && __ldcg(p.bad) != 0) return;  // offsets failed the check: read nothing
+    const int lane = threadIdx.x & 31;
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t Wn = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t base = __ldg(p.offsets);
+    const int64_t N = __ldg(p.offsets + p.nseg) - base;
+    int64_t E = (N + Wn - 1) / Wn;
+    E = ((E + PV - 1) / PV) * PV;
+    if (E < PV) E = PV;
+    const int64_t lo = base + (w * E < N ? w * E : N);
+    const int64_t hi = base + ((w + 1) * E < N ? (w + 1) * E : N);
+
+    // geometry of the piece: scalar head [lo, c0), vector body of nch chunks
+    // (last_ce elements in the last), scalar tail [.., hi)
+    const uintptr_t addr = reinterpret_cast<uintptr_t>(p.x) + (uintptr_t)lo * EB;
+    int64_t c0 = lo + (int64_t)(((uintptr_t)VB - addr % VB) % VB) / EB;
+    if (c0 > hi) c0 = hi;
+    const int64_t body = (hi - c0) / PV * PV;
+    const int nch = (int)((body + CE - 1) / CE);
+    const int last_ce = (int)(body - (int64_t)(nch - 1) * CE);
+
+    extern __shared__ __align__(1024) unsigned char seg_dsm[];
+    const int wib = threadIdx.x >> 5, nwib = blockDim.x >> 5, S = p.stages;
+    const uint32_t ring = smem_u32(seg_dsm) + (uint32_t)(wib * S) * CHUNK;
+    const uint32_t bars = smem_u32(seg_dsm) + (uint32_t)(nwib * S) * CHUNK + (uint32_t)(wib * S) * 8u;
+    // the strip table: word t describes strip t's boundaries of one offsets window
+    const uint32_t table =
+        smem_u32(seg_dsm) + (uint32_t)(nwib * S) * (CHUNK + 8u) + (uint32_t)(wib * kStripTableBytes);
+    // lane 0: copy chunk k of the body into ring stage st, if there is one
+    auto issue = [&](const unsigned char* src, int k, int st) {
+        if (k >= nch) return;
+        const uint32_t bytes = k == nch - 1 ? (uint32_t)last_ce * EB : CHUNK;
+        mbar_arrive_expect_tx(bars + 8u * st, bytes);
+        bulk_g2s(ring + (uint32_t)st * CHUNK, src, bytes, bars + 8u * st);
+    };
+    if (lane == 0) {
+        for (int st = 0; st < S; ++st) mbar_init(bars + 8u * st, 1);
+        mbar_fence_init();
+        for (int st = 0; st < S; ++st) issue(p.x + (c0 + (int64_t)st * CE) * EB, st, st);
+    }
+    __syncwarp();
+
+    // Stream state (warp-uniform).  The offsets window: lane k holds
+    // offsets[wb + k] in win and offsets[wb + 32 + k] in nxt (loaded one window
+    // ahead).  Entry kb is the end of the open segment, wb + kb - 1.
+    int64_t wb, win;
+    const int64_t at = N > 0 ? (int64_t)((float)(w * E) / (float)N * (float)p.nseg) : 0;
+    const int r0 = (int)(warp_search(p.offsets, p.nseg, base + w * E, at < p.nseg ? at : p.nseg, lane, wb, win) - wb);
+    int64_t nxt = (wb + 32 + lane <= p.nseg) ? __ldg(p.offsets + wb + 32 + lane) : INT64_MAX;
+    int64_t cur_start = __shfl_sync(0xffffffffu, win, r0);
+    // the open segment began in an earlier warp's piece (its true start is not needed)
+    bool cont = lo < hi && cur_start > lo;
+    if (cont) cur_start = lo;
+    int kb = cont ? r0 : r0 + 1;
+    int64_t cur_end = __shfl_sync(0xffffffffu, win, kb);
+    A acc = Op<A>::zero();  // this lane's part of the open segment
+    bool spread = false;    // acc is nonzero in lanes other than lane 0
+
+    auto next_window = [&]() {
+        win = nxt;
+        wb += 32;
+        kb = 0;
+        nxt = (wb + 32 + lane <= p.nseg) ? __ldg(p.offsets + wb + 32 + lane) : INT64_MAX;
+        if (wb + kAheadOffsets + lane <= p.nseg)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p.offsets + wb + kAheadOffsets + lane));
+    };
+    // this warp's piece of segment s, owned by an earlier warp; v in lane 0
+    auto emit_first = [&](int64_t s, A v) {
+        cont = false;
+        if (p.stage == kStageAtomic) {
+            if (lane == 0) seg_atomic(p, s, v);
+            return;
+        }
+        if (lane == 0) carry_store(p, p.carry_first, w, v);
+        if (p.stage == kStageLastBlock)
+            span_arrive<A>(p, s, (__ldg(p.offsets + s) - base) / E, (__ldg(p.offsets + s + 1) - 1 - base) / E, lane);
+    };
+    // the open segment's sum so far, in lane 0; acc restarts at zero
+    auto take_acc = [&]() {
+        const A v = spread ? warp_reduce(acc) : acc;
+        acc = Op<A>::zero();
+        spread = false;
+        return v;
+    };
+    // close the open segment (it ends inside the piece) and move to the next one
+    auto emit_advance = [&]() {
+        const A v = take_acc();
+        if (cont) emit_first(wb + kb - 1, v);
+        else if (lane == 0) seg_out(p, wb + kb - 1, v);
+        cur_start = cur_end;
+        if (++kb == 32) next_window();
+        cur_end = __shfl_sync(0xffffffffu, win, kb);
+    };
+    // scalar chunk [b0, b1), at most 32 elements: lane l holds element b0 + l
+    auto scalar_chunk = [&](int64_t b0, int64_t b1) {
+        if (b0 >= b1) return;
+        const int64_t idx = b0 + lane;
+        A one = Op<A>::zero();
+        if (idx < b1) acc_elem<DT>(one, p.x, idx);
+        for (;;) {
+            if (idx < b1 && idx >= cur_start && idx < cur_end) acc = Op<A>::add(acc, one);
+            if (cur_end > b0) spread = true;
+            if (cur_end >= b1) break;
+            emit_advance();
+        }
+    };
+
+    // Lane l reads vector j ^ sw of its strip at step j: eight consecutive lanes
+    // then hit eight different 16-byte bank groups (strips are a multiple of 32
+    // bytes apart, which in order is an up to 8-way conflict).
+    const int sw = (NV >= 8 ? lane : lane / (8 / NV)) & (NV - 1);
+
+    // elements [a, b) of the chunk in stage sb, a < b, summed by one lane, which
+    // starts at a vector of its own choosing (with equal lengths of a power of two
+    // the first ones would all lie on the same banks)
+    auto own_sum = [&](uint32_t sb, int a, int b) {
+        const uint32_t va = (unsigned)a / EV, vb = (unsigned)(b - 1) / EV;
+        const int nb = b - (int)vb * EV;  // elements of the last vector
+        uint32_t r[4];
+        if constexpr (kCompact) {
+            uint32_t i = va + ((uint32_t)lane & 7u);
+            if (i > vb) i = va;
+            VP v = VP::zero();
+#pragma unroll 1
+            for (uint32_t k = va; k <= vb; ++k) {
+                lds_vec(sb + 16u * i, r);
+                if (i == va) keep_from<EB>(r, a & (EV - 1));
+                if (i == vb) keep_below<EB>(r, nb);
+                v.add(VP::of(r));
+                if (++i > vb) i = va;
+            }
+            return v.total();
+        } else {  // the masked ends apart from the whole vectors between them
+            lds_vec(sb + 16u * va, r);
+            keep_from<EB>(r, a & (EV - 1));
+            if (va == vb) keep_below<EB>(r, nb);
+            VP v = VP::of(r);
+            if (va != vb) {
+                const uint32_t m = vb - va - 1;
+                uint32_t i = (uint32_t)lane & 7u;
+                if (i >= m) i = 0;
+                for (uint32_t n = 0; n < m; ++n) {
+                    lds_vec(sb + 16u * (va + 1u + i), r);
+                    v.add(VP::of(r));
+                    if (++i == m) i = 0;
+                }
+                lds_vec(sb + 16u * vb, r);
+                keep_below<EB>(r, nb);
+                v.add(VP::of(r));
+            }
+            return v.total();
+        }
+    };
+
+    // the chunk of `ce` elements from c0 in ring stage `sb`, zero-filled to CHUNK bytes
+    auto chunk = [&](int ce, uint32_t sb) {
+        const uint32_t strip = sb + (uint32_t)lane * (CHUNK / 32u);
+        const uint32_t v0 = strip + 16u * (uint32_t)sw;  // the strip is aligned to its size
+        if (cur_end >= c0 + ce) {  // no segment ends inside the chunk
+            VP v[2] = {VP::zero(), VP::zero()};
+#pragma unroll (UN / 2)
+            for (int j = 0; j < NV; j += 2) {
+                uint32_t r0[4], r1[4];
+                lds_vec(v0 ^ (16u * j), r0);
+                lds_vec(v0 ^ (16u * j + 16u), r1);
+                v[0].add(VP::of(r0));
+                v[1].add(VP::of(r1));
+            }
+            v[0].add(v[1]);
+            acc = Op<A>::add(acc, v[0].total());
+            spread = true;
+            return;
+        }
+        // Boundaries of the chunk, one offsets window at a time; positions
+        // relative to c0.  prev: the boundary before the window's first, -1 when
+        // the open segment began at c0 or before.
+        int prev = -1, rp, rpp;
+        bool is_b, short_only;
+        auto window = [&]() {
+            const int64_t ahead = win - c0;
+            rp = ahead < ce ? (int)ahead : 2 * CE;
+            is_b = lane >= kb && rp < ce;
+            rpp = __shfl_up_sync(0xffffffffu, rp, 1);  // the boundary before this lane's
+            if (lane == kb) rpp = prev;
+        };
+        // steps past the window's boundaries; true when more of the chunk's follow
+        auto advance = [&]() {
+            kb += __popc(__ballot_sync(0xffffffffu, is_b));
+            prev = __shfl_sync(0xffffffffu, rp, kb - 1);
+            if (kb < 32) return false;
+            next_window();
+            return __shfl_sync(0xffffffffu, win, 0) < c0 + ce;
+        };
+        // windows whose segments are all short: every lane sums the one that ends
+        // at its boundary, straight from shared memory
+        window();
+        short_only = true;
+        const int last = __shfl_sync(0xffffffffu, rp, 31);
+        if (last < ce) {  // the window after this one has a say too: mixing both ways in one chunk costs both
+            const int64_t ahead = nxt - c0;
+            const int np = ahead < ce ? (int)ahead : 2 * CE;
+            int npp = __shfl_up_sync(0xffffffffu, np, 1);
+            if (lane == 0) npp = last;
+                short_only = !__any_sync(0xffffffffu, np < ce && np - npp > kOwn);
+        }
+        while (short_only) {
+            const int from = rpp > 0 ? rpp : 0;
+            if (__any_sync(0xffffffffu, is_b && rp - from > kOwn)) break;
+            A v = Op<A>::zero();
+            if (is_b && rp > from) v = own_sum(sb, from, rp);
+            bool write = is_b;
+            if (prev < 0) {  // the first one: with what earlier chunks hold of it
+                const A before = Op<A>::shfl(take_acc(), 0);
+                if (lane == kb) v = Op<A>::add(before, v);
+                if (cont) {
+                    write = is_b && lane != kb;
+                    emit_first(wb + kb - 1, Op<A>::shfl(v, kb));
+                }
+            }
+            if (write) seg_out(p, wb + lane - 1, v);
+            if (advance()) {
+                window();
+                continue;
+            }
+            // the segment open at the chunk's end: [prev, CE), vectors spread over the lanes
+            VP t = VP::zero();
+            for (uint32_t k = (unsigned)prev / EV + lane; k < 32u * NV; k += 32u) {
+                uint32_t r[4];
+                lds_vec(sb + 16u * k, r);
+                if (k == (unsigned)prev / EV) keep_from<EB>(r, prev & (EV - 1));
+                t.add(VP::of(r));
+            }
+            acc = t.total();
+            spread = true;
+            cur_start = c0 + prev;
+            cur_end = __shfl_sync(0xffffffffu, win, kb);
+            return;
+        }
+        // the rest of the chunk by strips
+        const int begin = prev;  // >= 0: a boundary whose segment is closed already
+        int qf = SE, ql = SE;    // this lane's strip: first and last boundary (SE: none)
+        int64_t qseg = 0;        // the segment that ends at the first one
+        for (;;) {
+            asm volatile("st.shared.u32 [%0], %1;" ::"r"(table + 4u * lane), "r"(0xffffffffu) : "memory");
+            __syncwarp();
+            const int rpn = __shfl_down_sync(0xffffffffu, rp, 1);  // the boundary after this lane's
+            if (is_b) {
+                const int t = (int)((unsigned)rp / SE), q = (int)((unsigned)rp % SE);
+                if (rpp >= t * SE) {  // starts and ends inside strip t
+                    seg_out(p, wb + lane - 1, rp > rpp ? own_sum(sb, rpp, rp) : Op<A>::zero());
+                } else {  // the strip's first boundary
+                    const unsigned short e = (unsigned short)(q | (lane << 8));
+                    asm volatile("st.shared.u16 [%0], %1;" ::"r"(table + 4u * t), "h"(e) : "memory");
+                }
+                // the strip's last boundary in this window (a later window may hold one after it)
+                if (lane == 31 || rpn >= (t + 1) * SE) {
+                    const unsigned short e = (unsigned short)q;
+                    asm volatile("st.shared.u16 [%0], %1;" ::"r"(table + 4u * t + 2u), "h"(e) : "memory");
+                }
+            }
+            __syncwarp();
+            uint32_t e;
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(e) : "r"(table + 4u * lane) : "memory");
+            if ((e & 0xffffu) != 0xffffu) {
+                qf = (int)(e & 0xffu);
+                qseg = wb + (int)((e >> 8) & 0xffu) - 1;
+            }
+            if ((e >> 16) != 0xffffu) ql = (int)(e >> 16);
+            if (!advance()) break;
+            window();
+        }
+        cur_start = c0 + prev;
+        cur_end = __shfl_sync(0xffffffffu, win, kb);
+
+        bool closes = qf < SE;
+        if (begin >= 0 && lane == (int)((unsigned)begin / SE)) {
+            qf = begin & (SE - 1);  // the run from here on is new, and nothing is left to close
+            if (ql == SE) ql = qf;
+            closes = false;
+        }
+        const bool has_b = qf < SE;
+        const unsigned tmask = __ballot_sync(0xffffffffu, has_b);
+        const int vf = (int)((unsigned)qf / EV), vl = (int)((unsigned)ql / EV);  // NV when there is none
+        VP hv = VP::zero(), tv = VP::zero();
+#pragma unroll (UN)
+        for (int j = 0; j < NV; ++j) {
+            const int kv = j ^ sw;
+            uint32_t r[4];
+            lds_vec(v0 ^ (16u * j), r);
+            const VP v = VP::of(r);
+            if (kv < vf) hv.add(v);
+            if (kv > vl) tv.add(v);
+        }
+        if (has_b) {  // the boundary vectors
+            uint32_t r[4];
+            lds_vec(strip + 16u * vf, r);
+            keep_below<EB>(r, qf & (EV - 1));
+            hv.add(VP::of(r));
+            lds_vec(strip + 16u * vl, r);
+            keep_from<EB>(r, ql & (EV - 1));
+            tv.add(VP::of(r));
+        }
+        // the open segment of the chunks before enters at strip 0
+        A head = hv.total();
+        const A before = take_acc();
+        if (lane == 0) head = Op<A>::add(before, head);
+        // segmented inclusive scan of the open runs over the strips: before the
+        // step with distance d a lane's partial covers lanes [lane - d + 1,
+        // lane], and takes in the lanes before them unless one of its own holds
+        // a boundary, that is while d <= reach
+        const unsigned upto = tmask & ((2u << lane) - 1u);  // boundary lanes 0 .. lane (2 << 31 wraps to 0)
+        const int reach = upto ? lane - (31 - __clz(upto)) : lane;
+        A x = has_b ? tv.total() : head;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const A xo = Op<A>::shfl_up(x, d);
+            if (d <= reach) x = Op<A>::add(xo, x);
+        }
+        A closed = Op<A>::shfl_up(x, 1);  // the run open at the end of the strip before
+        closed = lane == 0 ? head : Op<A>::add(closed, head);
+        const A open_end = Op<A>::shfl(x, 31);
+        if (lane == 0) acc = open_end;
+        if (cont) {  // the first segment to end began in an earlier warp's piece
+            const int fl = __ffs(tmask) - 1;
+            emit_first(__shfl_sync(0xffffffffu, qseg, fl), Op<A>::shfl(closed, fl));
+            closes = closes && lane != fl;
+        }
+        if (closes) seg_out(p, qseg, closed);
+    };
+
+    int st = 0;
+    uint32_t par = 0;
+    bool bail = false;
+    const unsigned char* src = p.x + (c0 + (int64_t)S * CE) * EB;  // the next chunk to copy
+    scalar_chunk(lo, c0);
+    for (int k = 0; k < nch; ++k) {
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(bars + 8u * st, par, p.limit_ns))) {
+            if (lane == 0) {
+                atomicOr(p.err, kErrTimeout);
+                // leave no copy writing this CTA's shared memory: wait for the ones
+                // issued (chunks k .. k + S - 1), bounded separately (>= 1 s)
+                const uint64_t drain = p.limit_ns > 1000000000ull ? p.limit_ns : 1000000000ull;
+                for (int j = k; j < nch && j < k + S; ++j) {
+                    mbar_wait_bounded(bars + 8u * st, par, drain);
+                    if (++st == S) {
+                        st = 0;
+                        par ^= 1u;
+                    }
+                }
+            }
+            bail = true;
+            break;
+        }
+        const int ce = k == nch - 1 ? last_ce : CE;
+        const uint32_t sb = ring + (uint32_t)st * CHUNK;
+        if (ce < CE) {  // a short copy (the piece's last): zeros behind it
+            for (uint32_t b = (uint32_t)ce * EB + 16u * lane; b < CHUNK; b += 512u)
+                asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(sb + b), "r"(0) : "memory");
+            __syncwarp();
+        }
+        while (cur_end <= c0) emit_advance();
+        chunk(ce, sb);
+        __syncwarp();  // every lane has read the stage
+        if (lane == 0) {
+            fence_proxy_async_smem();
+            issue(src, k + S, st);
+        }
+        src += CHUNK;
+        c0 += ce;
+        if (++st == S) {
+            st = 0;
+            par ^= 1u;
+        }
+    }
+    int64_t spanning = -1;  // the owned segment that runs past this piece
+    if (!bail) {            // a timeout's results are void (SR_ERR_TIMEOUT): nothing left to finish
+        scalar_chunk(c0, hi);
+        const int64_t next_lo = (w == Wn - 1) ? INT64_MAX : base + (w + 1) * E;
         // the segment holding the piece's last element, then any (empty) segment
         // this warp owns that starts at or after hi
-        while (cur < p.nseg && cur_start < next_lo) emit_advance();
-    } else {
-        spanning = -1;  // results are void (SR_ERR_TIMEOUT); nothing left to finish
+        while (wb + kb <= p.nseg && cur_start < next_lo) {
+            if (cur_end <= hi || cont) {
+                emit_advance();
+                continue;
+            }
+            spanning = wb + kb - 1;  // owned, runs past this piece
+            const A v = take_acc();
+            if (p.stage == kStageAtomic) {
+                if (lane == 0) seg_atomic(p, spanning, v);
+            } else {
+                if (lane == 0) carry_store(p, p.carry_last, w, v);
+                if (p.stage == kStageLastBlock)
+                    span_arrive<A>(p, spanning, w, (cur_end - 1 - base) / E, lane);
+            }
+            break;  // the next segment starts in the next warp's piece
+        }
     }
 
     if (p.stage == kStageTwoKernel || p.stage == kStageGridSync) {
@@ -567,10 +1086,10 @@ __global__ void __launch_bounds__(256) seg_finish_kernel(const SegParams p, int6
 template <int DT, bool COMP, int VB, bool DENSE>
 inline const void* pick_seg(int unroll) {
     switch (unroll) {
-    case 1: return (const void*)seg_kernel<DT, COMP, VB, 1, DENSE, false>;
-    case 2: return (const void*)seg_kernel<DT, COMP, VB, 2, DENSE, false>;
-    case 4: return (const void*)seg_kernel<DT, COMP, VB, 4, DENSE, false>;
-    case 8: return DENSE ? nullptr : (const void*)seg_kernel<DT, COMP, VB, 8, false, false>;
+    case 1: return (const void*)seg_kernel<DT, COMP, VB, 1, DENSE>;
+    case 2: return (const void*)seg_kernel<DT, COMP, VB, 2, DENSE>;
+    case 4: return (const void*)seg_kernel<DT, COMP, VB, 4, DENSE>;
+    case 8: return DENSE ? nullptr : (const void*)seg_kernel<DT, COMP, VB, 8, false>;
     default: return nullptr;
     }
 }
@@ -578,9 +1097,9 @@ inline const void* pick_seg(int unroll) {
 template <int DT, bool COMP, int VB>
 inline const void* pick_seg_bulk(int unroll) {
     switch (unroll) {
-    case 2: return (const void*)seg_kernel<DT, COMP, VB, 2, false, true>;
-    case 4: return (const void*)seg_kernel<DT, COMP, VB, 4, false, true>;
-    case 8: return (const void*)seg_kernel<DT, COMP, VB, 8, false, true>;
+    case 2: return (const void*)seg_strip_kernel<DT, COMP, VB, 2>;
+    case 4: return (const void*)seg_strip_kernel<DT, COMP, VB, 4>;
+    case 8: return (const void*)seg_strip_kernel<DT, COMP, VB, 8>;
     default: return nullptr;
     }
 }

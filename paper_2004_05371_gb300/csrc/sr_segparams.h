@@ -15,6 +15,11 @@ constexpr int kErrQueueFull = 8;   // adaptive form: chunk queue overflow (never
 constexpr int64_t kAdaptQueueCap = 196608;       // chunk descriptors
 constexpr int64_t kAdaptChunkBytes = 64 << 10;   // smallest chunk (bytes of input)
 
+// TMA form: shared memory of one warp's strip table (one word per lane).  128
+// bytes fit beside every ring that fits a CTA's shared memory without it (the
+// tightest, 16 warps x 7 stages x 2 KiB, leaves 136 per warp).
+constexpr int kStripTableBytes = 128;
+
 // Kernel argument block of the segmented sum (sr_segmented_kernels.cuh).
 struct SegParams {
     const unsigned char* x;
