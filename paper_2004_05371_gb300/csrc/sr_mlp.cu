@@ -1,7 +1,7 @@
 // Small MLP cost model of the learned selector: in_dim -> hidden (ReLU) ->
 // hidden (ReLU) -> out_dim logits, softmax cross-entropy against soft target
 // distributions, trained with Adam.  All arithmetic runs in these kernels:
-//   mlp_grad_kernel   : forward + backward of a chunk of samples per CTA;
+//   mlp_grad_kernel   : forward + backward of tiles of eight samples per CTA;
 //                       every gradient entry is owned by one thread, and the
 //                       CTA's partial gradient is written to its own slot;
 //   mlp_update_kernel : sums the CTA partials in a fixed order (deterministic)
@@ -11,6 +11,7 @@
 //                       layer's dot products split over all 256 threads.
 // Parameter layout (row-major, one contiguous float array):
 //   W1[in][h], b1[h], W2[h][h], b2[h], W3[h][out], b3[out].
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -23,7 +24,6 @@ namespace {
 
 constexpr int kMaxIn = 32, kMaxH = 64, kMaxOut = 64;
 constexpr int kThreads = 256;
-constexpr int kSamplesPerCta = 16;
 
 struct MlpDims {
     int in, h, out;
@@ -46,140 +46,299 @@ MlpDims make_dims(int in, int h, int out) {
     return d;
 }
 
-// Shared-memory forward pass of one sample; returns nothing, fills h1, h2, z.
-__device__ __forceinline__ void forward_one(const MlpDims& d, const float* w, const float* x, float* h1, float* h2,
-                                            float* z) {
-    const int t = threadIdx.x;
-    if (t < d.h) {
-        float a = w[d.ob1 + t];
-        for (int i = 0; i < d.in; ++i) a = fmaf(x[i], w[d.oW1 + (int64_t)i * d.h + t], a);
-        h1[t] = a > 0.f ? a : 0.f;
-    }
-    __syncthreads();
-    if (t < d.h) {
-        float a = w[d.ob2 + t];
-        for (int j = 0; j < d.h; ++j) a = fmaf(h1[j], w[d.oW2 + (int64_t)j * d.h + t], a);
-        h2[t] = a > 0.f ? a : 0.f;
-    }
-    __syncthreads();
-    if (t < d.out) {
-        float a = w[d.ob3 + t];
-        for (int k = 0; k < d.h; ++k) a = fmaf(h2[k], w[d.oW3 + (int64_t)k * d.out + t], a);
-        z[t] = a;
-    }
-    __syncthreads();
+// Gradient kernel.  A batch is a few megaflops, so the step is bound by the
+// chain of dependent layers, not by throughput: with one sample at a time it
+// was some 10 block barriers and 60-long serial sums per sample, 16 samples in a
+// row (146 us a step of the 9-64-40 network at every batch up to 2048; now 9.8 us
+// to 256, 11.8 at 1000, 17.6 at 2048, two launches of some 3 and 6 us, bound by
+// shared-memory latency).  Here a CTA takes tiles of kTile
+// samples through each layer together: thread (column, half of the tile) sums
+// one column for four samples, so a weight is read once for four products, and
+// the weight gradients are outer products summed in registers over all tiles of
+// the CTA (thread: 4 rows x 8 columns).  The order of every sum over inputs and
+// over a tile's samples is that of one sample after the other.
+// Layout: weights with a row stride of 65 words (rows and columns are both read
+// by 32 lanes without bank conflicts); activations as [feature][kTile], 12 words
+// apart (eight consecutive features' float4 fall into different banks).
+constexpr int kGradThreads = 128;
+constexpr int kTile = 8;    // samples of a tile
+constexpr int kWLd = kMaxH + 1;
+constexpr int kALd = kTile + 4;
+
+struct GradSmem {  // offsets in floats
+    int w1, w2, w3, b1, b2, b3, x, h1, h2, z, dh2, dh1, loss, total;
+};
+__host__ __device__ inline GradSmem grad_smem(const MlpDims& d) {
+    GradSmem m;
+    int at = 0;
+    auto take = [&](int n) {
+        const int r = at;
+        at += (n + 3) / 4 * 4;
+        return r;
+    };
+    m.w1 = take(d.in * kWLd);
+    m.w2 = take(d.h * kWLd);
+    m.w3 = take(d.h * kWLd);
+    m.b1 = take(kMaxH);
+    m.b2 = take(kMaxH);
+    m.b3 = take(kMaxOut);
+    m.x = take(kMaxIn * kALd);
+    m.h1 = take(kMaxH * kALd);
+    m.h2 = take(kMaxH * kALd);
+    m.z = take(kMaxOut * kALd);  // logits, then their gradient
+    m.dh2 = take(kMaxH * kALd);
+    m.dh1 = take(kMaxH * kALd);
+    m.loss = take(kTile);
+    m.total = at;
+    return m;
 }
 
-__global__ void __launch_bounds__(kThreads) mlp_grad_kernel(MlpDims d, const float* __restrict__ params,
-                                                            const float* __restrict__ X, const float* __restrict__ Q,
-                                                            int B, float* __restrict__ partial,
-                                                            float* __restrict__ loss_partial) {
-    extern __shared__ float sm[];
-    float* w = sm;                // P
-    float* g = w + d.P;           // P
-    float* x = g + d.P;           // kMaxIn
-    float* h1 = x + kMaxIn;       // kMaxH
-    float* h2 = h1 + kMaxH;       // kMaxH
-    float* z = h2 + kMaxH;        // kMaxOut
-    float* dz = z + kMaxOut;      // kMaxOut
-    float* dh2 = dz + kMaxOut;    // kMaxH
-    float* dh1 = dh2 + kMaxH;     // kMaxH
-    __shared__ float s_loss;
-    const int t = threadIdx.x;
-    for (int64_t i = t; i < d.P; i += blockDim.x) {
-        w[i] = params[i];
-        g[i] = 0.f;
+// One float into shared memory, asynchronously (zero when !valid; src is not read then).
+__device__ __forceinline__ void copy_async(float* dst, const float* src, bool valid) {
+    const int bytes = valid ? 4 : 0;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(bytes) : "memory");
+}
+// Rows [0, rows) of a row-major matrix into shared memory, zero beyond `cols`:
+// all copies of the kernel's start are in flight together, one trip to L2.
+__device__ __forceinline__ void load_rows(float* dst, const float* __restrict__ src, int rows, int cols) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll 4
+    for (int r = warp; r < rows; r += kGradThreads / 32) {
+#pragma unroll
+        for (int c = lane; c < kMaxH; c += 32) copy_async(dst + r * kWLd + c, c < cols ? src + r * cols + c : src, c < cols);
     }
-    if (t == 0) s_loss = 0.f;
-    __syncthreads();
+}
+
+// acc[i] += sum_k W(k) * a[k][sg * 4 + i] over k < K; W(k) = w[k * step]
+__device__ __forceinline__ void dot4(float (&acc)[4], const float* w, int step, const float* a, int K) {
+#pragma unroll 16
+    for (int k = 0; k < K; ++k) {
+        const float wk = w[k * step];
+        const float4 v = *reinterpret_cast<const float4*>(a + k * kALd);
+        acc[0] = fmaf(v.x, wk, acc[0]);
+        acc[1] = fmaf(v.y, wk, acc[1]);
+        acc[2] = fmaf(v.z, wk, acc[2]);
+        acc[3] = fmaf(v.w, wk, acc[3]);
+    }
+}
+
+// g[j][c] += sum over the tile's samples of a[row_j][s] * b[col_c][s], rows
+// rg + 16 j, columns cg + 8 c.
+template <int NR>
+__device__ __forceinline__ void outer(float (&g)[NR][8], const float* a, const float* b, int rg, int cg) {
+#pragma unroll
+    for (int h = 0; h < kTile; h += 4) {
+        float4 u[NR];
+#pragma unroll
+        for (int j = 0; j < NR; ++j) u[j] = *reinterpret_cast<const float4*>(a + (rg + 16 * j) * kALd + h);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const float4 v = *reinterpret_cast<const float4*>(b + (cg + 8 * c) * kALd + h);
+#pragma unroll
+            for (int j = 0; j < NR; ++j) {
+                g[j][c] = fmaf(u[j].x, v.x, g[j][c]);
+                g[j][c] = fmaf(u[j].y, v.y, g[j][c]);
+                g[j][c] = fmaf(u[j].z, v.z, g[j][c]);
+                g[j][c] = fmaf(u[j].w, v.w, g[j][c]);
+            }
+        }
+    }
+}
+template <int NR>
+__device__ __forceinline__ void store_grad(float* out, const float (&g)[NR][8], int rows, int cols, int rg, int cg) {
+#pragma unroll
+    for (int j = 0; j < NR; ++j) {
+        const int r = rg + 16 * j;
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            if (r < rows && cg + 8 * c < cols) out[r * cols + cg + 8 * c] = g[j][c];
+    }
+}
+
+__global__ void __launch_bounds__(kGradThreads) mlp_grad_kernel(MlpDims d, const float* __restrict__ params,
+                                                                const float* __restrict__ X,
+                                                                const float* __restrict__ Q, int B,
+                                                                float* __restrict__ partial,
+                                                                float* __restrict__ loss_partial) {
+    extern __shared__ __align__(16) float sm[];
+    const GradSmem m = grad_smem(d);
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int col = t & 63, sg = t >> 6;      // forward and backward: a column, four samples
+    const int rg = t >> 3, cg = t & 7;        // weight gradients: rows rg + 16 j, columns cg + 8 c
+    grid_dependency_wait();  // the step before may have just written the parameters
+    allow_dependents();
+    load_rows(sm + m.w1, params + d.oW1, d.in, d.h);
+    load_rows(sm + m.w2, params + d.oW2, d.h, d.h);
+    load_rows(sm + m.w3, params + d.oW3, d.h, d.out);
+    if (t < kMaxH) {
+        copy_async(sm + m.b1 + t, params + (t < d.h ? d.ob1 + t : 0), t < d.h);
+        copy_async(sm + m.b2 + t, params + (t < d.h ? d.ob2 + t : 0), t < d.h);
+        copy_async(sm + m.b3 + t, params + (t < d.out ? d.ob3 + t : 0), t < d.out);
+    }
+    // rows past the network's own sizes are read by the outer products: zero them once
+    for (int i = t; i < m.loss - m.x; i += kGradThreads) sm[m.x + i] = 0.f;
+    float g1[2][8] = {}, g2[4][8] = {}, g3[4][8] = {};  // W1 (in <= 32), W2, W3
+    float gb[3] = {};                                   // thread t < 64: entry t of b1, b2, b3
+    float loss = 0.f;                                   // thread 0
     const float invB = 1.0f / (float)B;
-    const int b0 = blockIdx.x * kSamplesPerCta;
-    const int b1 = min(B, b0 + kSamplesPerCta);
-    for (int b = b0; b < b1; ++b) {
-        if (t < d.in) x[t] = X[(int64_t)b * d.in + t];
+    const int tiles = (B + kTile - 1) / kTile;
+    __syncthreads();
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int b0 = tile * kTile, nb = min(kTile, B - b0);
+        for (int i = t; i < kTile * d.in; i += kGradThreads) {
+            const int s = i / d.in, f = i - s * d.in;
+            sm[m.x + f * kALd + s] = s < nb ? X[(int64_t)b0 * d.in + i] : 0.f;
+        }
+        float q[2][2];  // this warp's two samples' targets, for the softmax below
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int s = 2 * warp + k;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int o = lane + 32 * h;
+                q[k][h] = (s < nb && o < d.out) ? Q[(int64_t)(b0 + s) * d.out + o] : 0.f;
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");  // the first tile: the weights
         __syncthreads();
-        forward_one(d, w, x, h1, h2, z);
-        // softmax cross-entropy (warp 0): dz = (p - q) / B, loss += -sum q log p
-        if (t < 32) {
-            float m = -INFINITY;
-            for (int o = t; o < d.out; o += 32) m = fmaxf(m, z[o]);
-            for (int off = 16; off; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-            float s = 0.f;
-            for (int o = t; o < d.out; o += 32) s += expf(z[o] - m);
-            for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-            const float lse = m + logf(s);
+        // one layer's column `col` for samples 4 sg .. 4 sg + 3; samples past the batch are zero
+        auto layer = [&](int w, int bias, int src, int K, int dst, bool relu) {
+            const float bv = sm[bias + col];
+            float a[4] = {bv, bv, bv, bv};
+            dot4(a, sm + w + col, kWLd, sm + src + sg * 4, K);
+            float4 r;
+            float* rv = reinterpret_cast<float*>(&r);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) rv[i] = (sg * 4 + i < nb && !(relu && !(a[i] > 0.f))) ? a[i] : 0.f;
+            *reinterpret_cast<float4*>(sm + dst + col * kALd + sg * 4) = r;
+            __syncthreads();
+        };
+        layer(m.w1, m.b1, m.x, d.in, m.h1, true);
+        layer(m.w2, m.b2, m.h1, d.h, m.h2, true);
+        layer(m.w3, m.b3, m.h2, d.h, m.z, false);
+        // softmax cross-entropy, two samples per warp: z becomes (p - q) / B
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int s = 2 * warp + k;
+            float z[2], mx = -INFINITY;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                z[h] = lane + 32 * h < d.out ? sm[m.z + (lane + 32 * h) * kALd + s] : -INFINITY;
+                mx = fmaxf(mx, z[h]);
+            }
+            for (int off = 16; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+            float e = 0.f;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) e += lane + 32 * h < d.out ? expf(z[h] - mx) : 0.f;
+            for (int off = 16; off; off >>= 1) e += __shfl_xor_sync(0xffffffffu, e, off);
+            const float lse = mx + logf(e);
             float l = 0.f;
-            for (int o = t; o < d.out; o += 32) {
-                const float q = Q[(int64_t)b * d.out + o];
-                const float p = expf(z[o] - lse);
-                dz[o] = (p - q) * invB;
-                l += q * (lse - z[o]);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int o = lane + 32 * h;
+                if (o < d.out) {
+                    sm[m.z + o * kALd + s] = s < nb ? (expf(z[h] - lse) - q[k][h]) * invB : 0.f;
+                    l += q[k][h] * (lse - z[h]);
+                }
             }
             for (int off = 16; off; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
-            if (t == 0) s_loss += l * invB;
+            if (lane == 0) sm[m.loss + s] = s < nb ? l * invB : 0.f;
         }
         __syncthreads();
-        // layer 3 gradients and dh2
-        if (t < d.h) {
-            float a = 0.f;
-            for (int o = 0; o < d.out; ++o) a = fmaf(w[d.oW3 + (int64_t)t * d.out + o], dz[o], a);
-            dh2[t] = h2[t] > 0.f ? a : 0.f;
+        // backward: row `col` of W for the tile's samples, masked by the activation's sign
+        auto back = [&](int w, int src, int K, int act, int dst) {
+            if (col < d.h) {
+                float a[4] = {0.f, 0.f, 0.f, 0.f};
+                dot4(a, sm + w + col * kWLd, 1, sm + src + sg * 4, K);
+                const float4 h = *reinterpret_cast<const float4*>(sm + act + col * kALd + sg * 4);
+                *reinterpret_cast<float4*>(sm + dst + col * kALd + sg * 4) =
+                    make_float4(h.x > 0.f ? a[0] : 0.f, h.y > 0.f ? a[1] : 0.f, h.z > 0.f ? a[2] : 0.f,
+                                h.w > 0.f ? a[3] : 0.f);
+            }
+        };
+        auto bias_grad = [&](float& g, int src) {
+            if (t < kMaxH) {
+#pragma unroll
+                for (int s = 0; s < kTile; ++s) g += sm[src + t * kALd + s];
+            }
+        };
+        back(m.w3, m.z, d.out, m.h2, m.dh2);
+        outer(g3, sm + m.h2, sm + m.z, rg, cg);
+        bias_grad(gb[2], m.z);
+        if (t == 0) {
+#pragma unroll
+            for (int s = 0; s < kTile; ++s) loss += sm[m.loss + s];
         }
-        for (int64_t i = t; i < (int64_t)d.h * d.out; i += blockDim.x) {
-            const int k = (int)(i / d.out), o = (int)(i % d.out);
-            g[d.oW3 + i] = fmaf(h2[k], dz[o], g[d.oW3 + i]);
-        }
-        if (t < d.out) g[d.ob3 + t] += dz[t];
         __syncthreads();
-        // layer 2 gradients and dh1
-        if (t < d.h) {
-            float a = 0.f;
-            for (int k = 0; k < d.h; ++k) a = fmaf(w[d.oW2 + (int64_t)t * d.h + k], dh2[k], a);
-            dh1[t] = h1[t] > 0.f ? a : 0.f;
-        }
-        for (int64_t i = t; i < (int64_t)d.h * d.h; i += blockDim.x) {
-            const int j = (int)(i / d.h), k = (int)(i % d.h);
-            g[d.oW2 + i] = fmaf(h1[j], dh2[k], g[d.oW2 + i]);
-        }
-        if (t < d.h) g[d.ob2 + t] += dh2[t];
+        back(m.w2, m.dh2, d.h, m.h1, m.dh1);
+        outer(g2, sm + m.h1, sm + m.dh2, rg, cg);
+        bias_grad(gb[1], m.dh2);
         __syncthreads();
-        // layer 1 gradients
-        for (int64_t i = t; i < (int64_t)d.in * d.h; i += blockDim.x) {
-            const int ii = (int)(i / d.h), j = (int)(i % d.h);
-            g[d.oW1 + i] = fmaf(x[ii], dh1[j], g[d.oW1 + i]);
-        }
-        if (t < d.h) g[d.ob1 + t] += dh1[t];
+        outer(g1, sm + m.x, sm + m.dh1, rg, cg);
+        bias_grad(gb[0], m.dh1);
         __syncthreads();
     }
     float* out = partial + (int64_t)blockIdx.x * d.P;
-    for (int64_t i = t; i < d.P; i += blockDim.x) out[i] = g[i];
-    if (t == 0) loss_partial[blockIdx.x] = s_loss;
+    store_grad(out + d.oW1, g1, d.in, d.h, rg, cg);
+    store_grad(out + d.oW2, g2, d.h, d.h, rg, cg);
+    store_grad(out + d.oW3, g3, d.h, d.out, rg, cg);
+    if (t < d.h) {
+        out[d.ob1 + t] = gb[0];
+        out[d.ob2 + t] = gb[1];
+    }
+    if (t < d.out) out[d.ob3 + t] = gb[2];
+    if (t == 0) loss_partial[blockIdx.x] = loss;
 }
 
-// Sum the per-CTA partials in CTA order, optionally export the gradient, and
-// (lr > 0) apply Adam: m = b1 m + (1-b1) g; v = b2 v + (1-b2) g^2;
+// Sum the per-CTA partials in a fixed order, optionally export the gradient,
+// and (lr > 0) apply Adam: m = b1 m + (1-b1) g; v = b2 v + (1-b2) g^2;
 // p -= lr * (m / (1 - b1^t)) / (sqrt(v / (1 - b2^t)) + eps).
-__global__ void mlp_update_kernel(int64_t P, int nparts, const float* __restrict__ partial,
-                                  const float* __restrict__ loss_partial, float* __restrict__ params,
-                                  float* __restrict__ m, float* __restrict__ v, float* __restrict__ grad_out,
-                                  float* __restrict__ loss_out, float lr, float b1, float b2, float eps, float c1,
-                                  float c2) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0 && loss_out) {
-        float l = 0.f;
-        for (int k = 0; k < nparts; ++k) l += loss_partial[k];
-        *loss_out = l;
+// A CTA takes 32 parameters; its warp k sums the partials k, k + 8, ..., warp 0
+// adds the eight sums in order (one thread per parameter walked all partials
+// alone: with 128 of them, 128 dependent adds behind as many loads).
+constexpr int kUpdGroups = 8;
+
+__global__ void __launch_bounds__(32 * kUpdGroups)
+    mlp_update_kernel(int64_t P, int nparts, const float* __restrict__ partial, const float* __restrict__ loss_partial,
+                      float* params, float* m, float* v, float* __restrict__ grad_out, float* __restrict__ loss_out,
+                      float lr, float b1, float b2, float eps, float c1, float c2) {
+    __shared__ float part[kUpdGroups][33];
+    const int lane = threadIdx.x & 31, group = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane;
+    // The state is read before the wait (from L2): the gradient kernel this one
+    // follows waited for the update before it, so nothing in flight writes it.
+    float mi = 0.f, vi = 0.f, pi = 0.f;
+    if (group == 0 && i < P && lr > 0.f) {
+        mi = __ldcg(m + i);
+        vi = __ldcg(v + i);
+        pi = __ldcg(params + i);
     }
-    if (i >= P) return;
+    grid_dependency_wait();  // the partials are written
+    allow_dependents();
+    float s = 0.f;
+    if (i < P) {
+#pragma unroll 4
+        for (int k = group; k < nparts; k += kUpdGroups) s += partial[(int64_t)k * P + i];
+    }
+    part[group][lane] = s;
+    float l = 0.f;
+    if (blockIdx.x == 0 && group == 1 && loss_out) {
+        for (int k = lane; k < nparts; k += 32) l += loss_partial[k];
+        for (int off = 16; off; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+        if (lane == 0) *loss_out = l;
+    }
+    __syncthreads();
+    if (group != 0 || i >= P) return;
     float gsum = 0.f;
-    for (int k = 0; k < nparts; ++k) gsum += partial[(int64_t)k * P + i];
+#pragma unroll
+    for (int k = 0; k < kUpdGroups; ++k) gsum += part[k][lane];
     if (grad_out) grad_out[i] = gsum;
     if (lr > 0.f) {
-        const float mi = b1 * m[i] + (1.f - b1) * gsum;
-        const float vi = b2 * v[i] + (1.f - b2) * gsum * gsum;
+        mi = b1 * mi + (1.f - b1) * gsum;
+        vi = b2 * vi + (1.f - b2) * gsum * gsum;
         m[i] = mi;
         v[i] = vi;
-        params[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+        params[i] = pi - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
     }
 }
 
@@ -360,7 +519,11 @@ int sr_mlp_train_step(sr_mlp h, const float* X, const float* Q, int batch, float
                       sr_stream_t stream) {
     if (!h || !X || !Q || batch < 1 || !(lr >= 0.f)) return SR_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    const int parts = (batch + kSamplesPerCta - 1) / kSamplesPerCta;
+    int st = SR_OK;
+    const DeviceInfo* di = current_device(&st);
+    if (!di) return st;
+    // one tile of samples per CTA up to two CTAs per SM, then several
+    const int parts = (int)std::min<int64_t>(((int64_t)batch + kTile - 1) / kTile, 2 * di->sms);
     cudaError_t e;
     if (parts > h->max_parts) {
         cudaFree(h->partial);
@@ -375,20 +538,34 @@ int sr_mlp_train_step(sr_mlp h, const float* X, const float* Q, int batch, float
         }
         h->max_parts = parts;
     }
-    const size_t smem = sizeof(float) * (size_t)(2 * h->d.P + kMaxIn + 4 * kMaxH + 2 * kMaxOut);
-    int st = prepare_function((const void*)mlp_grad_kernel, smem, false);
+    const size_t smem = sizeof(float) * (size_t)grad_smem(h->d).total;
+    st = prepare_function((const void*)mlp_grad_kernel, smem, false);
     if (st != SR_OK) return st;
-    mlp_grad_kernel<<<parts, kThreads, smem, s>>>(h->d, h->params, X, Q, batch, h->partial, h->loss_partial);
-    e = cudaGetLastError();
+    // programmatic stream serialisation: each kernel is scheduled while the one
+    // before it drains and waits for it before its first global read
+    cudaLaunchAttribute pdl[1];
+    pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t lc;
+    std::memset(&lc, 0, sizeof lc);
+    lc.gridDim = dim3((unsigned)parts);
+    lc.blockDim = dim3(kGradThreads);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = s;
+    lc.attrs = pdl;
+    lc.numAttrs = 1;
+    e = cudaLaunchKernelEx(&lc, mlp_grad_kernel, h->d, (const float*)h->params, X, Q, batch, h->partial,
+                           h->loss_partial);
     if (e != cudaSuccess) return status_from_cuda(e);
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     if (lr > 0.f) h->step += 1;
     const float c1 = lr > 0.f ? 1.f - powf(b1, (float)h->step) : 1.f;
     const float c2 = lr > 0.f ? 1.f - powf(b2, (float)h->step) : 1.f;
-    const int blocks = (int)((h->d.P + 255) / 256);
-    mlp_update_kernel<<<blocks, 256, 0, s>>>(h->d.P, parts, h->partial, h->loss_partial, h->params, h->m, h->v, grad,
-                                             loss, lr, b1, b2, eps, c1, c2);
-    e = cudaGetLastError();
+    lc.gridDim = dim3((unsigned)((h->d.P + 31) / 32));
+    lc.blockDim = dim3(32 * kUpdGroups);
+    lc.dynamicSmemBytes = 0;
+    e = cudaLaunchKernelEx(&lc, mlp_update_kernel, h->d.P, parts, (const float*)h->partial,
+                           (const float*)h->loss_partial, h->params, h->m, h->v, grad, loss, lr, b1, b2, eps, c1, c2);
     return e == cudaSuccess ? SR_OK : status_from_cuda(e);
 }
 
