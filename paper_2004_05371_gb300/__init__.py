@@ -223,9 +223,33 @@ def check(status: int, what: str = ""):
         raise SRError(status, what)
 
 
+# The pieces of torch a call needs, bound at the first one: a small sum takes
+# 2 us on the device, and looking these up on every call took longer.
+_torch = None
+_DTYPE_CODES = {}
+_raw_stream = _device_index = None
+
+
+def _bind_torch():
+    global _torch, _raw_stream, _device_index
+    import torch
+    _DTYPE_CODES.update({torch.float32: F32, torch.int32: I32, torch.bfloat16: BF16, torch.uint8: FP8E4M3})
+    fp8 = getattr(torch, "float8_e4m3fn", None)
+    if fp8 is not None:
+        _DTYPE_CODES[fp8] = FP8E4M3
+    _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    _device_index = getattr(torch._C, "_cuda_getDevice", None)
+    _torch = torch
+    return torch
+
+
 def _stream(stream):
     if stream is None:
-        import torch
+        torch = _torch or _bind_torch()
+        # the handle of the current device's current stream; without the raw
+        # getters, or before CUDA is up, through the public call (3 us)
+        if _raw_stream is not None and _device_index is not None and torch.cuda.is_initialized():
+            return _raw_stream(_device_index())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
@@ -233,18 +257,16 @@ def _stream(stream):
 
 
 def dtype_code(t) -> int:
-    import torch
-    m = {torch.float32: F32, torch.int32: I32, torch.bfloat16: BF16, torch.uint8: FP8E4M3}
-    fp8 = getattr(torch, "float8_e4m3fn", None)
-    if fp8 is not None:
-        m[fp8] = FP8E4M3
-    if t.dtype not in m:
+    if _torch is None:
+        _bind_torch()
+    code = _DTYPE_CODES.get(t.dtype)
+    if code is None:
         raise TypeError("unsupported dtype %s" % t.dtype)
-    return m[t.dtype]
+    return code
 
 
 def out_dtype(dtype: int, variant: int):
-    import torch
+    torch = _torch or _bind_torch()
     if dtype == I32:
         return torch.int64
     return torch.float64 if variant & F_FP64_COMBINE else torch.float32
@@ -261,8 +283,7 @@ def make_config(variant=AUTO, **kw) -> Config:
 def reduce_sum_ptr(x_ptr: int, n: int, dtype: int, out_ptr: int, config: Config = None, stream=None) -> int:
     """Raw call of sr_reduce_sum_ex; returns the status (no raise)."""
     cfg = ctypes.byref(config) if config is not None else None
-    return lib().sr_reduce_sum_ex(ctypes.c_void_p(x_ptr), int(n), int(dtype), ctypes.c_void_p(out_ptr), cfg,
-                                  ctypes.c_void_p(_stream(stream)))
+    return (_lib or load()).sr_reduce_sum_ex(x_ptr, int(n), int(dtype), out_ptr, cfg, _stream(stream))
 
 
 def reduce_sum_noalloc_ptr(x_ptr: int, n: int, dtype: int, out_ptr: int, config: Config = None,
@@ -286,14 +307,13 @@ def reduce_sum(x, variant: int = AUTO, out=None, config: Config = None, stream=N
     Returns a 0-dim CUDA tensor (int64 for int32 input, float64 with
     F_FP64_COMBINE, float32 otherwise).  uint8 input is read as FP8 E4M3 codes.
     """
-    import torch
     if not x.is_cuda or not x.is_contiguous():
         raise ValueError("x must be a contiguous CUDA tensor")
     dt = dtype_code(x)
     if config is None:
         config = make_config(variant, **cfg_fields)
     if out is None:
-        out = torch.empty((), dtype=out_dtype(dt, config.variant), device=x.device)
+        out = _torch.empty((), dtype=out_dtype(dt, config.variant), device=x.device)
     st = reduce_sum_ptr(x.data_ptr(), x.numel(), dt, out.data_ptr(), config, stream)
     check(st, "sr_reduce_sum_ex")
     return out
@@ -303,9 +323,8 @@ def reduce_sum_segmented_ptr(x_ptr: int, offsets_ptr: int, nseg: int, dtype: int
                              config: Config = None, stream=None) -> int:
     """Raw call of sr_reduce_sum_segmented_ex; returns the status (no raise)."""
     cfg = ctypes.byref(config) if config is not None else None
-    return lib().sr_reduce_sum_segmented_ex(ctypes.c_void_p(x_ptr), ctypes.c_void_p(offsets_ptr), int(nseg),
-                                            int(dtype), ctypes.c_void_p(out_ptr), cfg,
-                                            ctypes.c_void_p(_stream(stream)))
+    return (_lib or load()).sr_reduce_sum_segmented_ex(x_ptr, offsets_ptr, int(nseg), int(dtype), out_ptr, cfg,
+                                                       _stream(stream))
 
 
 def reduce_sum_segmented_checked_ptr(x_ptr: int, n_elems: int, offsets_ptr: int, nseg: int, dtype: int,
@@ -323,7 +342,7 @@ def reduce_sum_segmented(x, offsets, variant: int = AUTO, out=None, config: Conf
                          **cfg_fields):
     """Per-segment sums of a CUDA tensor over int64 CSR offsets (CUDA tensor of
     nseg + 1 entries).  Returns a CUDA tensor of nseg results."""
-    import torch
+    torch = _torch or _bind_torch()
     if not (x.is_cuda and offsets.is_cuda and x.is_contiguous() and offsets.is_contiguous()):
         raise ValueError("x and offsets must be contiguous CUDA tensors")
     if offsets.dtype != torch.int64:
@@ -448,16 +467,15 @@ class MLP:
     def train_step(self, X, Q, lr: float, loss=None, grad=None, stream=None):
         """X, Q: CUDA float32 tensors [B, in] / [B, out]; loss: CUDA float32
         scalar tensor (optional); grad: CUDA float32 [P] (optional)."""
-        B = X.shape[0]
-        check(lib().sr_mlp_train_step(self.h, ctypes.c_void_p(X.data_ptr()), ctypes.c_void_p(Q.data_ptr()), B,
-                                      float(lr), ctypes.c_void_p(loss.data_ptr() if loss is not None else None),
-                                      ctypes.c_void_p(grad.data_ptr() if grad is not None else None),
-                                      ctypes.c_void_p(_stream(stream))), "sr_mlp_train_step")
+        check(lib().sr_mlp_train_step(self.h, X.data_ptr(), Q.data_ptr(), X.shape[0], float(lr),
+                                      loss.data_ptr() if loss is not None else None,
+                                      grad.data_ptr() if grad is not None else None, _stream(stream)),
+              "sr_mlp_train_step")
 
     def predict(self, X, cls, logits=None, stream=None):
-        check(lib().sr_mlp_predict(self.h, ctypes.c_void_p(X.data_ptr()), X.shape[0], ctypes.c_void_p(cls.data_ptr()),
-                                   ctypes.c_void_p(logits.data_ptr() if logits is not None else None),
-                                   ctypes.c_void_p(_stream(stream))), "sr_mlp_predict")
+        check(lib().sr_mlp_predict(self.h, X.data_ptr(), X.shape[0], cls.data_ptr(),
+                                   logits.data_ptr() if logits is not None else None, _stream(stream)),
+              "sr_mlp_predict")
 
     def close(self):
         if self.h:
