@@ -19,7 +19,7 @@ namespace sr {
 //   seg          : segmented-reduction carries
 constexpr int kMaxUnits = 65536;
 constexpr size_t kSlotBytes = 16;
-constexpr size_t kSegBytes = 8u << 20;  // also holds the adaptive form's chunk queue (sr_segparams.h)
+constexpr size_t kSegBytes = 3u << 20;
 // Segmented carries: tickets (4 B), last_seg (8 B), carry_first and
 // carry_last (16 B each) per warp: 44 B x 65536 warps = 2.75 MiB <= kSegBytes.
 constexpr int64_t kSegMaxWarps = 65536;
@@ -69,6 +69,7 @@ struct SegPlan {
     bool comp = false, fp64 = false, dense = false, bulk = false, warp = false, lane = false, adapt = false;
     int vec = 16, unroll = 4, block = 256, grid = 0;
     int stages = 0;
+    int ring = 0;     // TMA form: stages the kernel runs with (see plan_tma)
     size_t smem = 0;  // dynamic shared memory of the TMA form
     int64_t warps = 0;
     float scale = 1.f;

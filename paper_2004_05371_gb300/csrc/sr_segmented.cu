@@ -37,45 +37,65 @@ constexpr int kSegFormFlags =
 // atomically.  2^21 segments of 16: 61.8 us with the 16 MiB zeroed, 54.6 with
 // tickets; 90,000 of 16: 9.6 against 11.7.
 constexpr int64_t kSegZeroMax = 1 << 19;
+constexpr int kAdaptMaxCtasPerSm = 4;  // adaptive form: largest grid it takes, in CTAs per SM
 constexpr int64_t kSegBulkMin = 32768;  // segments from which the default shape is the TMA form
 
-const void* seg_adapt_kernel(int dtype, bool comp, int vec, int unroll) {
-    switch (dtype) {
-    case SR_F32: return seg_adapt_f32(comp, vec, unroll);
-    case SR_I32: return seg_adapt_i32(comp, vec, unroll);
-    case SR_BF16: return seg_adapt_bf16(comp, vec, unroll);
-    case SR_FP8E4M3: return seg_adapt_fp8(comp, vec, unroll);
-    default: return nullptr;
-    }
-}
-
-bool seg_kernels(int dtype, bool comp, int vec, int unroll, bool dense, bool bulk, bool warp, bool lane,
-                 const void** main, const void** fin) {
+// The kernels of the forms other than the TMA one.
+bool seg_kernels(int dtype, bool comp, int vec, int unroll, bool dense, bool warp, bool lane, const void** main,
+                 const void** fin) {
     const void* (*ldg)(bool, int, int, const void**) = nullptr;
     const void* (*den)(bool, int, int) = nullptr;
-    const void* (*tma)(bool, int, int) = nullptr;
     const void* (*wrp)(bool, int, int) = nullptr;
     const void* (*lan)(bool, int, int) = nullptr;
     switch (dtype) {
-    case SR_F32: ldg = seg_ldg_f32; den = seg_dense_f32; tma = seg_tma_f32; wrp = seg_warp_f32; lan = seg_lane_f32; break;
-    case SR_I32: ldg = seg_ldg_i32; den = seg_dense_i32; tma = seg_tma_i32; wrp = seg_warp_i32; lan = seg_lane_i32; break;
-    case SR_BF16:
-        ldg = seg_ldg_bf16; den = seg_dense_bf16; tma = seg_tma_bf16; wrp = seg_warp_bf16; lan = seg_lane_bf16;
-        break;
-    case SR_FP8E4M3:
-        ldg = seg_ldg_fp8; den = seg_dense_fp8; tma = seg_tma_fp8; wrp = seg_warp_fp8; lan = seg_lane_fp8;
-        break;
+    case SR_F32: ldg = seg_ldg_f32; den = seg_dense_f32; wrp = seg_warp_f32; lan = seg_lane_f32; break;
+    case SR_I32: ldg = seg_ldg_i32; den = seg_dense_i32; wrp = seg_warp_i32; lan = seg_lane_i32; break;
+    case SR_BF16: ldg = seg_ldg_bf16; den = seg_dense_bf16; wrp = seg_warp_bf16; lan = seg_lane_bf16; break;
+    case SR_FP8E4M3: ldg = seg_ldg_fp8; den = seg_dense_fp8; wrp = seg_warp_fp8; lan = seg_lane_fp8; break;
     default: return false;
     }
     if (warp || lane) {  // one kernel, nothing to finish
         *fin = nullptr;
-        *main = (dense || bulk || (warp && lane)) ? nullptr : (warp ? wrp(comp, vec, unroll) : lan(comp, vec, unroll));
+        *main = warp ? wrp(comp, vec, unroll) : lan(comp, vec, unroll);
         return *main != nullptr;
     }
     const void* plain = ldg(comp, vec, unroll, fin);  // also sets the second kernel
-    if (bulk) *main = dense ? nullptr : tma(comp, vec, unroll);
-    else *main = dense ? den(comp, vec, unroll) : plain;
+    *main = dense ? den(comp, vec, unroll) : plain;
     return *main != nullptr;
+}
+
+// The TMA form's kernel for p (block and stages set) with chunks of `unroll`
+// rows of 32 `vec`-byte vectors; its second kernel, shared memory (per warp:
+// stages of a chunk and an mbarrier each, and the strip table) and resident CTAs.
+int plan_tma(SegPlan& p, int vec, int unroll, const DeviceInfo& d, int* resident) {
+    switch (p.dtype) {
+    case SR_F32: p.main = seg_tma_f32(p.comp, vec, unroll); seg_ldg_f32(p.comp, vec, unroll, &p.fin); break;
+    case SR_I32: p.main = seg_tma_i32(p.comp, vec, unroll); seg_ldg_i32(p.comp, vec, unroll, &p.fin); break;
+    case SR_BF16: p.main = seg_tma_bf16(p.comp, vec, unroll); seg_ldg_bf16(p.comp, vec, unroll, &p.fin); break;
+    default: p.main = seg_tma_fp8(p.comp, vec, unroll); seg_ldg_fp8(p.comp, vec, unroll, &p.fin); break;
+    }
+    if (!p.main) return SR_ERR_UNSUPPORTED;
+    const size_t ring = (size_t)(p.block / 32) * p.stages * ((size_t)unroll * 32 * vec + 8);
+    p.ring = p.stages;
+    p.smem = ring + (size_t)(p.block / 32) * kStripTableBytes;
+    if (p.smem > (size_t)d.smem_per_block_optin) return SR_ERR_LAUNCH;
+    int st = prepare_function(p.main, p.smem, false);
+    if (st != SR_OK) return st;
+    st = blocks_per_sm(d, p.main, p.block, p.smem, resident);
+    if (st != SR_OK) return st;
+    if (p.stages > 2) {
+        // a few shapes fill the SM so closely that the tables would cost a CTA:
+        // they take the place of one stage there
+        int bare = 0;
+        st = blocks_per_sm(d, p.main, p.block, ring, &bare);
+        if (st != SR_OK) return st;
+        if (bare > *resident) {
+            *resident = bare;
+            p.ring = p.stages - 1;
+            p.smem = ring;
+        }
+    }
+    return *resident < 1 ? SR_ERR_LAUNCH : SR_OK;
 }
 }  // namespace
 
@@ -140,26 +160,26 @@ int seg_plan(int64_t nseg, int dtype, const sr_config& c, const DeviceInfo& d, S
     }
     p.adapt = (c.variant & SR_F_ADAPTIVE_SEGMENTS) != 0;
     if (p.adapt) {
-        // one cooperative launch of the resident number of 256-thread CTAs;
-        // phase 1 at the warp form's shape (16-byte vectors, 2 per lane)
+        // Any layout: the TMA form at its default shape, finished by tickets
+        // (deterministic).  It balances the warps by elements whatever the
+        // lengths, and resolves short and long segments alike; against the
+        // device-side partition into lanes, lane groups and queued chunks it
+        // replaced (~2^28 elements): 4M lognormal f32 366 -> 200 us, 10,000
+        // lognormal 196 -> 162, 16M x 16 246 -> 229; 4M x 39 lognormal bf16 154
+        // -> 115.  The form's nominal shape is all a caller may name.
         if ((c.vec_bytes && c.vec_bytes != 16) || (c.unroll && c.unroll != 2) ||
             (c.block_threads && c.block_threads != 256))
             return SR_ERR_UNSUPPORTED;
+        if (c.grid > (int64_t)kAdaptMaxCtasPerSm * d.sms) return SR_ERR_LAUNCH;
+        p.block = 256;
+        p.stages = 2;
+        int resident = 0;
+        int st = plan_tma(p, 32, 4, d, &resident);
+        if (st != SR_OK) return st;
         p.vec = 16;
         p.unroll = 2;
-        p.block = 256;
-        p.main = seg_adapt_kernel(dtype, p.comp, p.vec, p.unroll);
-        p.fin = nullptr;
-        if (!p.main) return SR_ERR_UNSUPPORTED;
-        int st = prepare_function(p.main, 0, false);
-        if (st != SR_OK) return st;
-        int resident = 0;
-        st = blocks_per_sm(d, p.main, p.block, 0, &resident);
-        if (st != SR_OK) return st;
-        if (resident < 1) return SR_ERR_LAUNCH;
-        int64_t grid = c.grid ? c.grid : (int64_t)resident * d.sms;
-        if (grid > (int64_t)resident * d.sms) return SR_ERR_LAUNCH;  // could not be co-resident
-        p.grid = (int)std::max<int64_t>(1, grid);
+        const int64_t grid = c.grid ? c.grid : (int64_t)resident * d.sms;
+        p.grid = (int)std::max<int64_t>(1, std::min<int64_t>(grid, kSegMaxWarps / (p.block / 32)));
         p.warps = (int64_t)p.grid * (p.block / 32);
         *out = p;
         return SR_OK;
@@ -174,20 +194,19 @@ int seg_plan(int64_t nseg, int dtype, const sr_config& c, const DeviceInfo& d, S
     // 10,000 it is 1-3 % behind.
     const bool shape_given = c.vec_bytes || c.unroll || c.block_threads || c.stages;
     p.bulk = (c.variant & SR_F_BULK) != 0 || (!shape_given && !p.dense && !p.warp && !p.lane && nseg >= kSegBulkMin);
-    if (p.bulk) {  // per warp: stages x (unroll rows of 32 vectors + one mbarrier), and the strip table
+    int st, resident = 0;
+    if (p.bulk) {
         if (!c.unroll) p.unroll = 4;
         p.stages = c.stages ? c.stages : 2;
-        p.smem = (size_t)(p.block / 32) * (p.stages * ((size_t)p.unroll * 32 * p.vec + 8) + kStripTableBytes);
-        if (p.smem > (size_t)d.smem_per_block_optin) return SR_ERR_LAUNCH;
+        st = plan_tma(p, p.vec, p.unroll, d, &resident);
+        if (st != SR_OK) return st;
+    } else {
+        if (!seg_kernels(dtype, p.comp, p.vec, p.unroll, p.dense, p.warp, p.lane, &p.main, &p.fin))
+            return SR_ERR_UNSUPPORTED;
+        st = blocks_per_sm(d, p.main, p.block, 0, &resident);
+        if (st != SR_OK) return st;
+        if (resident < 1) return SR_ERR_LAUNCH;
     }
-    if (!seg_kernels(dtype, p.comp, p.vec, p.unroll, p.dense, p.bulk, p.warp, p.lane, &p.main, &p.fin))
-        return SR_ERR_UNSUPPORTED;
-    int st = prepare_function(p.main, p.smem, false);
-    if (st != SR_OK) return st;
-    int resident = 0;
-    st = blocks_per_sm(d, p.main, p.block, p.smem, &resident);
-    if (st != SR_OK) return st;
-    if (resident < 1) return SR_ERR_LAUNCH;
     int per_sm = c.ctas_per_sm ? std::min(c.ctas_per_sm, resident) : resident;
     int64_t grid = c.grid ? c.grid : (int64_t)d.sms * per_sm;
     grid = std::min<int64_t>(grid, kSegMaxWarps / (p.block / 32));
@@ -235,27 +254,13 @@ int seg_launch(const void* x, const int64_t* offsets, void* out, const SegPlan& 
     kp.carry_last = ws.seg + (size_t)kSegMaxWarps * 28;
     kp.err = ws.err;
     kp.scale = p.scale;
-    kp.stages = p.stages;
+    kp.stages = p.ring;
     kp.limit_ns = spin_limit_ns();
     kp.bad = check ? ws.check : nullptr;
-    kp.stage = p.stage;
+    kp.stage = p.adapt ? SR_LAST_BLOCK : p.stage;  // the adaptive form ignores the stage bits
     kp.fp64 = p.fp64 ? 1 : 0;
     cudaError_t e;
-    if (p.adapt) {
-        // the chunk queue: counters at the head of the tickets (the last warp
-        // of each launch resets them to zero), arrays after the tickets
-        SegQueue kq;
-        kq.ctr = reinterpret_cast<unsigned int*>(ws.seg);
-        unsigned char* q = ws.seg + (size_t)kSegMaxWarps * 4;
-        kq.desc = reinterpret_cast<long long*>(q);
-        kq.part = q + (size_t)kAdaptQueueCap * 16;
-        kq.tick = reinterpret_cast<unsigned int*>(q + (size_t)kAdaptQueueCap * 32);
-        kq.cap = kAdaptQueueCap;
-        void* aargs[] = {&kp, &kq};
-        e = cudaLaunchCooperativeKernel(p.main, dim3(p.grid), dim3(p.block), aargs, 0, s);
-        return e == cudaSuccess ? SR_OK : status_from_cuda(e);
-    }
-    if (p.stage == SR_ATOMIC && !p.warp && !p.lane) {
+    if (kp.stage == SR_ATOMIC && !p.warp && !p.lane) {
         const size_t ob = (p.dtype == SR_I32 || p.fp64) ? 8 : 4;
         const int zs = launch_zero(out, ob * (size_t)p.nseg, s);
         if (zs != SR_OK) return zs;
@@ -272,7 +277,7 @@ int seg_launch(const void* x, const int64_t* offsets, void* out, const SegPlan& 
     lc.stream = s;
     lc.attrs = pdl;
     lc.numAttrs = 1;
-    if (p.stage == SR_GRID_SYNC && !p.warp && !p.lane) {
+    if (kp.stage == SR_GRID_SYNC && !p.warp && !p.lane) {
         e = cudaLaunchCooperativeKernel(p.main, dim3(p.grid), dim3(p.block), args, p.smem, s);
     } else {
         lc.gridDim = dim3(p.grid);
@@ -282,7 +287,7 @@ int seg_launch(const void* x, const int64_t* offsets, void* out, const SegPlan& 
         lc.dynamicSmemBytes = 0;
     }
     if (e != cudaSuccess) return status_from_cuda(e);
-    if (p.stage == SR_TWO_KERNEL && !p.warp && !p.lane) {
+    if (kp.stage == SR_TWO_KERNEL && !p.warp && !p.lane) {
         int64_t wn = p.warps;
         int pv = p.vec / elem_size(p.dtype);
         void* fargs[] = {&kp, &wn, &pv};

@@ -8,12 +8,6 @@
 namespace sr {
 
 constexpr int kErrBadOffsets = 4;  // the checked entry found offsets it may not read with
-constexpr int kErrQueueFull = 8;   // adaptive form: chunk queue overflow (never by construction)
-
-// Adaptive form: the chunk queue in the segmented workspace, after the
-// flat split's tickets (which must stay zero between launches).
-constexpr int64_t kAdaptQueueCap = 196608;       // chunk descriptors
-constexpr int64_t kAdaptChunkBytes = 64 << 10;   // smallest chunk (bytes of input)
 
 // TMA form: shared memory of one warp's strip table (one word per lane).  128
 // bytes fit beside every ring that fits a CTA's shared memory without it (the
@@ -39,18 +33,6 @@ struct SegParams {
     const int* bad;             // checked entry: nonzero = offsets invalid, read nothing (else NULL)
 };
 
-// The adaptive form's chunk queue (see sr_segmented_kernels.cuh), a second
-// kernel parameter of that form only: the other segmented kernels keep their
-// argument block as it is (with these fields in it the flat split's code
-// generation changed and it ran 7 % slower).
-struct SegQueue {
-    unsigned int* ctr;          // [0] chunks queued, [1] next chunk to take, [2] warps done; zero between launches
-    long long* desc;            // 2 per chunk: segment, (chunk index << 32) | chunks of the segment
-    unsigned char* part;        // 16-byte partial per chunk
-    unsigned int* tick;         // per segment, at its first chunk: chunks finished
-    int64_t cap;                // chunk capacity
-};
-
 // Per-dtype segmented kernel selection, one function per kernel family and
 // dtype (each in its own translation unit): the LDG form (which also returns
 // the two-kernel form's second kernel), the dense variant, the TMA form.
@@ -71,11 +53,6 @@ const void* seg_warp_f32(bool comp, int vec, int unroll);
 const void* seg_warp_i32(bool comp, int vec, int unroll);
 const void* seg_warp_bf16(bool comp, int vec, int unroll);
 const void* seg_warp_fp8(bool comp, int vec, int unroll);
-// The adaptive form (mixed layouts, one cooperative launch), same unit.
-const void* seg_adapt_f32(bool comp, int vec, int unroll);
-const void* seg_adapt_i32(bool comp, int vec, int unroll);
-const void* seg_adapt_bf16(bool comp, int vec, int unroll);
-const void* seg_adapt_fp8(bool comp, int vec, int unroll);
 // The lane-per-segment form, in the same translation unit.
 const void* seg_lane_f32(bool comp, int vec, int unroll);
 const void* seg_lane_i32(bool comp, int vec, int unroll);

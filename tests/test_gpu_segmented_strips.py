@@ -101,3 +101,16 @@ def test_infinities_and_nans_stay_in_their_segment(sr):
         else:
             seg = x[off[s]:off[s + 1]].astype(np.float64)
             assert abs(got[s] - seg.sum()) <= 4 * EPS32 * np.abs(seg).sum(), s
+
+
+def test_ring_that_fills_the_sm(sr):
+    """A ring that two CTAs per SM just hold: the strip tables take a stage's
+    place, and a grid.sync() grid of two CTAs per SM still runs."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    off = workloads.segment_offsets(3000, 1 << 22, seed=3, median=512, sigma=1.5, lo=0, hi=1 << 16)
+    x = workloads.uniform_i32(int(off[-1]), seed=3)
+    for shape in ({"vec_bytes": 16, "unroll": 4, "stages": 7, "block_threads": 256},
+                  {"vec_bytes": 32, "unroll": 4, "stages": 4, "block_threads": 224}):
+        got = sr.reduce_sum_segmented(torch.from_numpy(x).cuda(), torch.from_numpy(off).cuda(),
+                                      config=sr.make_config(sr.GRID_SYNC | BULK, grid=2 * sms, **shape)).cpu().numpy()
+        assert np.array_equal(got, oracle.segsum_i32(x, off)), shape
