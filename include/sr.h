@@ -282,8 +282,8 @@ int sr_plan(int64_t n, int dtype, const sr_config* cfg, sr_config* resolved);
  * finished by the configured grid stage: SR_TWO_KERNEL, SR_GRID_SYNC,
  * SR_LAST_BLOCK (per-segment tickets; the SR_AUTO default for floating-point
  * inputs and from 2^19 segments) or SR_ATOMIC (out zeroed first; FP order not
- * deterministic; the SR_AUTO default for SR_I32 below 2^19 segments, whose
- * int64 sums are exact in any order).  All other forms are deterministic.
+ * deterministic; otherwise the SR_AUTO default for SR_I32, whose int64 sums
+ * are exact in any order).  All other forms are deterministic.
  * Load path: rows of 16/32-byte vectors loaded into registers (LDG), or with
  * SR_F_BULK each warp streams its piece through its own ring of `stages`
  * (2..8, default 2) chunks of `unroll` rows (2, 4 or 8; default 4) in shared
@@ -291,7 +291,9 @@ int sr_plan(int64_t n, int dtype, const sr_config* cfg, sr_config* resolved);
  * ends once per chunk and so also suits short segments; every wait bounded, an
  * expired one reported as SR_ERR_TIMEOUT by sr_stream_status).  Without an
  * explicit shape (vec_bytes, unroll, block_threads and stages all 0) calls
- * with 32768 or more segments take the TMA form, fewer the LDG one.
+ * with 32768 or more segments take the TMA form, fewer the LDG one — or, from
+ * 4096 segments, with no stage, grid or ctas_per_sm asked for either, the form of
+ * SR_F_ADAPTIVE_SEGMENTS.
  * With SR_F_WARP_SEGMENTS whole segments go to single warps instead, with
  * SR_F_LANE_SEGMENTS to single threads (see the flags): no segment is split,
  * the stage bits are ignored and the results are deterministic.  With

@@ -38,6 +38,7 @@ constexpr int kSegFormFlags =
 // tickets; 90,000 of 16: 9.6 against 11.7.
 constexpr int64_t kSegZeroMax = 1 << 19;
 constexpr int kAdaptMaxCtasPerSm = 4;  // adaptive form: largest grid it takes, in CTAs per SM
+constexpr int64_t kSegAdaptMin = 4096;  // segments from which the default is the adaptive form
 constexpr int64_t kSegBulkMin = 32768;  // segments from which the default shape is the TMA form
 
 // The kernels of the forms other than the TMA one.
@@ -158,7 +159,17 @@ int seg_plan(int64_t nseg, int dtype, const sr_config& c, const DeviceInfo& d, S
         p.vec = c.vec_bytes ? c.vec_bytes : 16;
         p.unroll = c.unroll ? c.unroll : 2;
     }
-    p.adapt = (c.variant & SR_F_ADAPTIVE_SEGMENTS) != 0;
+    // With nothing asked for, kSegAdaptMin or more segments (below kSegBulkMin)
+    // take the adaptive form: the LDG kernel pays for every segment end with a
+    // masked row and a warp reduction (20,000 lognormal segments of 2000 BF16
+    // values 48.6 us against 21.2; 14,454 of 445 f32 24.4 against 11.9; 10,000 of
+    // 26,844 f32 159 against 158).  With fewer, each segment spans many warps and the
+    // LDG kernel's shorter start wins (1000 of 1000 int32 5.7 us against 10.0; 2000
+    // of 400 f32 8.5 against 9.7; 3000 of 50 f32 8.8 against 8.5).
+    const bool shape_given = c.vec_bytes || c.unroll || c.block_threads || c.stages;
+    p.adapt = (c.variant & SR_F_ADAPTIVE_SEGMENTS) != 0 ||
+              (!shape_given && !c.grid && !c.ctas_per_sm && nseg >= kSegAdaptMin && nseg < kSegBulkMin &&
+               !(c.variant & (SR_STAGE_MASK | kSegFormFlags)));
     if (p.adapt) {
         // Any layout: the TMA form at its default shape, finished by tickets
         // (deterministic).  It balances the warps by elements whatever the
@@ -171,6 +182,7 @@ int seg_plan(int64_t nseg, int dtype, const sr_config& c, const DeviceInfo& d, S
             (c.block_threads && c.block_threads != 256))
             return SR_ERR_UNSUPPORTED;
         if (c.grid > (int64_t)kAdaptMaxCtasPerSm * d.sms) return SR_ERR_LAUNCH;
+        p.stage = SR_LAST_BLOCK;  // the stage bits are ignored
         p.block = 256;
         p.stages = 2;
         int resident = 0;
@@ -192,7 +204,6 @@ int seg_plan(int64_t nseg, int dtype, const sr_config& c, const DeviceInfo& d, S
     // form, which resolves segment ends once per chunk: from 100,000 to 16M
     // segments of ~2^28 elements it takes 164-229 us, the LDG default 192-3361; at
     // 10,000 it is 1-3 % behind.
-    const bool shape_given = c.vec_bytes || c.unroll || c.block_threads || c.stages;
     p.bulk = (c.variant & SR_F_BULK) != 0 || (!shape_given && !p.dense && !p.warp && !p.lane && nseg >= kSegBulkMin);
     int st, resident = 0;
     if (p.bulk) {
@@ -257,10 +268,10 @@ int seg_launch(const void* x, const int64_t* offsets, void* out, const SegPlan& 
     kp.stages = p.ring;
     kp.limit_ns = spin_limit_ns();
     kp.bad = check ? ws.check : nullptr;
-    kp.stage = p.adapt ? SR_LAST_BLOCK : p.stage;  // the adaptive form ignores the stage bits
+    kp.stage = p.stage;
     kp.fp64 = p.fp64 ? 1 : 0;
     cudaError_t e;
-    if (kp.stage == SR_ATOMIC && !p.warp && !p.lane) {
+    if (p.stage == SR_ATOMIC && !p.warp && !p.lane) {
         const size_t ob = (p.dtype == SR_I32 || p.fp64) ? 8 : 4;
         const int zs = launch_zero(out, ob * (size_t)p.nseg, s);
         if (zs != SR_OK) return zs;
@@ -277,7 +288,7 @@ int seg_launch(const void* x, const int64_t* offsets, void* out, const SegPlan& 
     lc.stream = s;
     lc.attrs = pdl;
     lc.numAttrs = 1;
-    if (kp.stage == SR_GRID_SYNC && !p.warp && !p.lane) {
+    if (p.stage == SR_GRID_SYNC && !p.warp && !p.lane) {
         e = cudaLaunchCooperativeKernel(p.main, dim3(p.grid), dim3(p.block), args, p.smem, s);
     } else {
         lc.gridDim = dim3(p.grid);
@@ -287,10 +298,11 @@ int seg_launch(const void* x, const int64_t* offsets, void* out, const SegPlan& 
         lc.dynamicSmemBytes = 0;
     }
     if (e != cudaSuccess) return status_from_cuda(e);
-    if (kp.stage == SR_TWO_KERNEL && !p.warp && !p.lane) {
+    if (p.stage == SR_TWO_KERNEL && !p.warp && !p.lane) {
         int64_t wn = p.warps;
         int pv = p.vec / elem_size(p.dtype);
-        void* fargs[] = {&kp, &wn, &pv};
+        int e_min = p.bulk ? p.unroll * 32 * pv / kPieceParts : pv;  // the first kernel's smallest piece
+        void* fargs[] = {&kp, &wn, &pv, &e_min};
         lc.gridDim = dim3((unsigned)((p.warps * 32 + 255) / 256));
         lc.blockDim = dim3(256);
         e = cudaLaunchKernelExC(&lc, p.fin, fargs);

@@ -197,11 +197,20 @@ template <class P> __device__ __forceinline__ P carry_load(const unsigned char* 
 // warp calls; fixed order, so the result does not depend on which warp runs it).
 template <class P> __device__ __forceinline__ void finish_span_typed(const SegParams& p, int64_t s, int64_t w_o,
                                                                      int64_t w_e, int lane) {
-    P acc = Op<P>::zero();
-    for (int64_t w = w_o + 1 + lane; w <= w_e; w += 32) acc = Op<P>::add(acc, carry_load<P>(p.carry_first, w));
+    P first = Op<P>::zero(), acc = Op<P>::zero();
+    if (lane == 0) first = carry_load<P>(p.carry_last, w_o);
+    int64_t w = w_o + 1 + lane;
+    for (; w + 7 * 32 <= w_e; w += 8 * 32) {  // eight loads in flight: a long segment has thousands of carries
+        P c[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) c[k] = carry_load<P>(p.carry_first, w + 32 * k);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) acc = Op<P>::add(acc, c[k]);
+    }
+    for (; w <= w_e; w += 32) acc = Op<P>::add(acc, carry_load<P>(p.carry_first, w));
     acc = warp_reduce(acc);
     if (lane == 0) {
-        P total = Op<P>::add(carry_load<P>(p.carry_last, w_o), acc);
+        P total = Op<P>::add(first, acc);
         if constexpr (std::is_same<P, double>::value) seg_out_d(p, s, total);
         else seg_out(p, s, total);
     }
@@ -653,7 +662,7 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
     const int64_t N = __ldg(p.offsets + p.nseg) - base;
     int64_t E = (N + Wn - 1) / Wn;
     E = ((E + PV - 1) / PV) * PV;
-    if (E < PV) E = PV;
+    if (E < CE / kPieceParts) E = CE / kPieceParts;
     const int64_t lo = base + (w * E < N ? w * E : N);
     const int64_t hi = base + ((w + 1) * E < N ? (w + 1) * E : N);
 
@@ -1062,7 +1071,7 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
 
 // Second kernel of the two-kernel form: one warp per first-kernel warp.
 template <int DT, bool COMP>
-__global__ void __launch_bounds__(256) seg_finish_kernel(const SegParams p, int64_t Wn, int PV) {
+__global__ void __launch_bounds__(256) seg_finish_kernel(const SegParams p, int64_t Wn, int PV, int e_min) {
     using A = typename Acc<DT, COMP>::T;
     grid_dependency_wait();  // the implicit barrier: every first-kernel warp has finished
     allow_dependents();
@@ -1076,7 +1085,7 @@ __global__ void __launch_bounds__(256) seg_finish_kernel(const SegParams p, int6
     const int64_t N = __ldg(p.offsets + p.nseg) - base;
     int64_t E = (N + Wn - 1) / Wn;  // the first kernel's piece size
     E = ((E + PV - 1) / PV) * PV;
-    if (E < PV) E = PV;
+    if (E < e_min) E = e_min;
     const int64_t end = __ldg(p.offsets + s + 1);
     finish_span<A>(p, s, w, (end - 1 - base) / E, lane);
 }
