@@ -30,6 +30,7 @@ struct KParams {
     int64_t body_bytes;       // bulk path: nvec * 16
     int64_t ntiles;           // bulk path: ceil(body_bytes / tile_bytes)
     uint64_t limit_ns;        // bound on every device-side wait
+    int prefetch;             // input larger than L2: see reduce_ldg_kernel
 };
 
 struct KernelSet {

@@ -216,6 +216,18 @@ template <int DT, bool COMP, int VB, int UNROLL>
 __global__ void __launch_bounds__(1024) reduce_ldg_kernel(const KParams p) {
     using A = typename Acc<DT, COMP>::T;
     constexpr int W = VB / 4;
+    // Large inputs: the CTA's first batch is fetched into L2 while the kernel before
+    // still drains.  Nothing is read here, and L2 is where both kernels' accesses
+    // meet, so data that kernel has yet to write arrives all the same.
+    if (p.prefetch && threadIdx.x == 0) {
+#pragma unroll
+        for (int u = 0; u < UNROLL; ++u) {
+            const int64_t i0 = ((int64_t)u * gridDim.x + blockIdx.x) * blockDim.x;
+            if (i0 < p.nvec)
+                prefetch_l2(p.x + p.head * ElemBytes<DT>::v + i0 * VB,
+                            (uint32_t)min((int64_t)blockDim.x, p.nvec - i0) * VB);
+        }
+    }
     grid_dependency_wait();
     allow_dependents();
     A acc[W];
@@ -295,6 +307,13 @@ __global__ void __launch_bounds__(1024) reduce_bulk_kernel(const KParams p) {
         }
         mbar_fence_init();
     }
+    const unsigned char* body = p.x + p.head * ElemBytes<DT>::v;
+    if (p.prefetch && threadIdx.x == 32) {  // the ring's first tiles, as in reduce_ldg_kernel
+        for (int s = 0; s < S; ++s) {
+            const int64_t off = ((int64_t)blockIdx.x + (int64_t)s * gridDim.x) * p.tile_bytes;
+            if (off < p.body_bytes) prefetch_l2(body + off, (uint32_t)min((int64_t)p.tile_bytes, p.body_bytes - off));
+        }
+    }
     grid_dependency_wait();  // shared-memory set-up above overlaps the previous kernel
     allow_dependents();
     __syncthreads();
@@ -302,7 +321,6 @@ __global__ void __launch_bounds__(1024) reduce_bulk_kernel(const KParams p) {
     const int64_t my_tiles = p.ntiles > (int64_t)blockIdx.x
                                  ? (p.ntiles - 1 - (int64_t)blockIdx.x) / gridDim.x + 1
                                  : 0;
-    const unsigned char* body = p.x + p.head * ElemBytes<DT>::v;
     A acc[4];
 #pragma unroll
     for (int w = 0; w < 4; ++w) acc[w] = Op<A>::zero();
@@ -430,8 +448,11 @@ __global__ void __launch_bounds__(1024) reduce_bulk_kernel(const KParams p) {
 
 // ---------------------------------------------- two-kernel second stage
 template <class P> __global__ void __launch_bounds__(1024) reduce_final_kernel(const KParams p) {
+    // A large input's next main kernel may be scheduled while this call's still
+    // drains (it waits for this kernel, which waits for that one): its CTAs prefetch.
+    if (p.prefetch) allow_dependents();
     grid_dependency_wait();  // the implicit barrier: every unit's partial is written
-    allow_dependents();
+    if (!p.prefetch) allow_dependents();
     reduce_slots<P>(p);
 }
 
