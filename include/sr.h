@@ -222,15 +222,16 @@ int sr_reduce_sum(const void* x, int64_t n, int dtype, void* out, int variant,
                   sr_stream_t stream);
 
 /* End-to-end form: x and out are HOST pointers (x preferably page-locked, e.g.
- * cudaHostAlloc / cudaHostRegister, so copies run asynchronously).  The input
- * is copied to the device in 64 MiB chunks through two library-owned staging
+ * cudaHostAlloc / cudaHostRegister, so copies run asynchronously).  With stage
+ * SR_AUTO a page-locked array of at most 128 MiB is read in place, as with
+ * SR_F_HOST_DIRECT; otherwise the input is copied to the device in 64 MiB chunks through two library-owned staging
  * buffers on two copy streams, each chunk reduced on `stream` while the next
  * one is copied (the chunk units' partials go to disjoint workspace slots),
- * one final kernel combines all partials in order, and the result is copied
- * back to *out.  Blocks until the result is in *out.  cfg: NULL, or stage
+ * and one final kernel combines all partials in order.  The result comes back
+ * through page-locked memory of the library's.  Blocks until the result is in *out.  cfg: NULL, or stage
  * SR_AUTO / SR_TWO_KERNEL with optional SR_F_KAHAN / SR_F_FP64_COMBINE and
  * launch-shape fields; other stages or SR_F_BULK -> SR_ERR_UNSUPPORTED.
- * The first call on a stream allocates the staging buffers (128 MiB).
+ * The first call that copies allocates the stream's staging buffers (128 MiB).
  * With SR_F_HOST_DIRECT there is no staging: one reduction (LDG path, stage
  * SR_LAST_BLOCK) reads x through its device mapping; SR_ERR_UNSUPPORTED when x
  * is neither page-locked nor accessible as pageable memory on this device.
