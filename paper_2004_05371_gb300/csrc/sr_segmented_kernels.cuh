@@ -73,9 +73,12 @@ __device__ __forceinline__ int64_t warp_lower_bound(const int64_t* off, int64_t 
 // and the answer r lies in [wb, wb + 30], so offsets[r] and offsets[r + 1] are
 // in the window.  The first probe spreads the lanes at power-of-two distances
 // around `guess`, the answer for equal segments: for layouts near it that is
-// one round of loads instead of log32(nseg) (whole warp calls).
+// one round of loads instead of log32(nseg) (whole warp calls).  `meanwhile` runs
+// when the last round is on its way: bulk traffic belongs there, since earlier
+// rounds would queue behind it.
+template <class F>
 __device__ __forceinline__ int64_t warp_search(const int64_t* off, int64_t nseg, int64_t key, int64_t guess, int lane,
-                                               int64_t& wb, int64_t& win) {
+                                               int64_t& wb, int64_t& win, F&& meanwhile) {
     int64_t lo = 0, hi = nseg;  // the answer is in [lo, hi]
     if (nseg > 30) {
         const int64_t i = lane < 16 ? guess - (1 << (15 - lane)) : guess + (1 << (lane - 16)) - 1;
@@ -103,6 +106,7 @@ __device__ __forceinline__ int64_t warp_search(const int64_t* off, int64_t nseg,
     }
     wb = lo;
     win = (lo + lane <= nseg) ? __ldg(off + lo + lane) : INT64_MAX;
+    meanwhile();
     return lo + __ffs(__ballot_sync(0xffffffffu, lo + lane >= hi || win >= key)) - 1;
 }
 
@@ -689,19 +693,24 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
         mbar_arrive_expect_tx(bars + 8u * st, bytes);
         bulk_g2s(ring + (uint32_t)st * CHUNK, src, bytes, bars + 8u * st);
     };
-    if (lane == 0) {
-        for (int st = 0; st < S; ++st) mbar_init(bars + 8u * st, 1);
-        mbar_fence_init();
-        for (int st = 0; st < S; ++st) issue(p.x + (c0 + (int64_t)st * CE) * EB, st, st);
-    }
-    __syncwarp();
+    // the ring's first copies (24 warps' rings are 30 MB for the chip: issued before
+    // the search they held the searching warps up to 8 us, now 4)
+    auto fill = [&]() {
+        if (lane == 0) {
+            for (int st = 0; st < S; ++st) mbar_init(bars + 8u * st, 1);
+            mbar_fence_init();
+            for (int st = 0; st < S; ++st) issue(p.x + (c0 + (int64_t)st * CE) * EB, st, st);
+        }
+        __syncwarp();
+    };
 
     // Stream state (warp-uniform).  The offsets window: lane k holds
     // offsets[wb + k] in win and offsets[wb + 32 + k] in nxt (loaded one window
     // ahead).  Entry kb is the end of the open segment, wb + kb - 1.
     int64_t wb, win;
     const int64_t at = N > 0 ? (int64_t)((float)(w * E) / (float)N * (float)p.nseg) : 0;
-    const int r0 = (int)(warp_search(p.offsets, p.nseg, base + w * E, at < p.nseg ? at : p.nseg, lane, wb, win) - wb);
+    const int r0 =
+        (int)(warp_search(p.offsets, p.nseg, base + w * E, at < p.nseg ? at : p.nseg, lane, wb, win, fill) - wb);
     int64_t nxt = (wb + 32 + lane <= p.nseg) ? __ldg(p.offsets + wb + 32 + lane) : INT64_MAX;
     int64_t cur_start = __shfl_sync(0xffffffffu, win, r0);
     // the open segment began in an earlier warp's piece (its true start is not needed)
