@@ -551,7 +551,8 @@ __global__ void __launch_bounds__(512, 1) seg_kernel(const SegParams p) {
 // are resident with two 4 KiB stages each: 16 warps of 112 registers took 4 %
 // less on long segments and 8-12 % more on short ones.
 
-// Sum of the elements in one 16-byte vector (four 32-bit words).
+// Sum of the elements in one 16-byte vector (four 32-bit words); compensated
+// binary32 and BF16 go through PackedPairs (below) instead.
 template <int DT, class A> __device__ __forceinline__ A vec_total(const uint32_t (&r)[4]) {
     if constexpr (DT == kDtI32) {
         long long s = (long long)(int)r[0];
@@ -562,14 +563,6 @@ template <int DT, class A> __device__ __forceinline__ A vec_total(const uint32_t
         const float v = AccVec<kDtFP8, float, 4>::vec_sum(r);  // 16 values: exact
         if constexpr (std::is_same<A, Pair>::value) return Pair{v, 0.f};
         else return v;
-    } else if constexpr (std::is_same<A, Pair>::value) {
-        Pair t[4];
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-            if constexpr (DT == kDtF32) t[w] = Pair{__uint_as_float(r[w]), 0.f};
-            else two_sum(__uint_as_float(r[w] << 16), __uint_as_float(r[w] & 0xffff0000u), t[w].s, t[w].c);
-        }
-        return Op<Pair>::add(Op<Pair>::add(t[0], t[1]), Op<Pair>::add(t[2], t[3]));
     } else if constexpr (DT == kDtBF16) {
         const float a = bf16_hi_add(r[1], bf16_lo_add(r[1], bf16_hi_add(r[0], __uint_as_float(r[0] << 16))));
         const float b = bf16_hi_add(r[3], bf16_lo_add(r[3], bf16_hi_add(r[2], __uint_as_float(r[2] << 16))));
@@ -606,6 +599,57 @@ template <> struct VecPart<kDtF32, float> {
     }
     __device__ __forceinline__ void add(const VecPart& b) { *this = sum(x, y, b.x, b.y); }
     __device__ __forceinline__ float total() const { return __fadd_rn(x, y); }
+};
+
+// Compensated binary32 and BF16: two (sum, correction) pairs in packed registers.
+// Each TwoSum (Knuth's, each half rounded like the scalar form) takes six packed
+// instructions for two pairs: a vector costs 14 (f32) or 28 (BF16) instead of 28 or 56.
+__device__ __forceinline__ void two_sum_packed(float ax, float ay, float bx, float by, float& sx, float& sy,
+                                               float& ex, float& ey) {
+    asm("{ .reg .b64 a, b, t, bp, ap, d1, d2, e;\n"
+        " mov.b64 a, {%4, %5};\n mov.b64 b, {%6, %7};\n"
+        " add.rn.f32x2 t, a, b;\n sub.rn.f32x2 bp, t, a;\n sub.rn.f32x2 ap, t, bp;\n"
+        " sub.rn.f32x2 d1, a, ap;\n sub.rn.f32x2 d2, b, bp;\n add.rn.f32x2 e, d1, d2;\n"
+        " mov.b64 {%0, %1}, t;\n mov.b64 {%2, %3}, e; }"
+        : "=f"(sx), "=f"(sy), "=f"(ex), "=f"(ey)
+        : "f"(ax), "f"(ay), "f"(bx), "f"(by));
+}
+struct PackedPairs {
+    float sx, sy, cx, cy;
+    __device__ __forceinline__ static PackedPairs zero() { return PackedPairs{0.f, 0.f, 0.f, 0.f}; }
+    __device__ __forceinline__ static PackedPairs of_sum(float ax, float ay, float bx, float by) {
+        PackedPairs t;
+        two_sum_packed(ax, ay, bx, by, t.sx, t.sy, t.cx, t.cy);
+        return t;
+    }
+    __device__ __forceinline__ void add(const PackedPairs& b) {
+        float ex, ey;
+        two_sum_packed(sx, sy, b.sx, b.sy, sx, sy, ex, ey);
+        VecPart<kDtF32, float> c = VecPart<kDtF32, float>::sum(cx, cy, b.cx, b.cy);
+        c = VecPart<kDtF32, float>::sum(c.x, c.y, ex, ey);
+        cx = c.x;
+        cy = c.y;
+    }
+    __device__ __forceinline__ Pair total() const { return Op<Pair>::add(Pair{sx, cx}, Pair{sy, cy}); }
+};
+template <> struct VecPart<kDtF32, Pair> : PackedPairs {
+    __device__ __forceinline__ static VecPart zero() { return VecPart{PackedPairs::zero()}; }
+    __device__ __forceinline__ static VecPart of(const uint32_t (&r)[4]) {
+        return VecPart{of_sum(__uint_as_float(r[0]), __uint_as_float(r[1]), __uint_as_float(r[2]),
+                              __uint_as_float(r[3]))};
+    }
+};
+template <> struct VecPart<kDtBF16, Pair> : PackedPairs {
+    __device__ __forceinline__ static VecPart zero() { return VecPart{PackedPairs::zero()}; }
+    __device__ __forceinline__ static PackedPairs two_words(uint32_t a, uint32_t b) {
+        return of_sum(__uint_as_float(a << 16), __uint_as_float(b << 16), __uint_as_float(a & 0xffff0000u),
+                      __uint_as_float(b & 0xffff0000u));
+    }
+    __device__ __forceinline__ static VecPart of(const uint32_t (&r)[4]) {
+        PackedPairs t = two_words(r[0], r[1]);
+        t.add(two_words(r[2], r[3]));
+        return VecPart{t};
+    }
 };
 
 // The low n bits (n <= 0: none, n >= 32: all).
