@@ -49,24 +49,25 @@ MlpDims make_dims(int in, int h, int out) {
 // Gradient kernel.  A batch is a few megaflops, so the step is bound by the
 // chain of dependent layers, not by throughput: with one sample at a time it
 // was some 10 block barriers and 60-long serial sums per sample, 16 samples in a
-// row (146 us a step of the 9-64-40 network at every batch up to 2048; now 9.8 us
-// to 256, 11.8 at 1000, 17.6 at 2048, two launches of some 3 and 6 us, bound by
-// shared-memory latency).  Here a CTA takes tiles of kTile
-// samples through each layer together: thread (column, half of the tile) sums
-// one column for four samples, so a weight is read once for four products, and
-// the weight gradients are outer products summed in registers over all tiles of
-// the CTA (thread: 4 rows x 8 columns).  The order of every sum over inputs and
-// over a tile's samples is that of one sample after the other.
+// row (146 us a step of the 9-64-40 network at every batch up to 2048; now 9.1 us
+// to 256, 10.4 at 1000, 15.9 at 2048, in two launches, bound by shared-memory
+// latency).  Here a CTA takes tiles of kTile
+// samples through each layer together: thread (column, half of the tile, half of
+// the inputs) sums one column for four samples, so a weight is read once for four
+// products; the two halves of the inputs meet in shared memory.  The weight
+// gradients are outer products summed in registers over all tiles of the CTA
+// (thread: 2 rows x 8 columns), the tile's samples in order.  With 128 threads and
+// whole columns the same step took 9.8, 11.3 and 16.4 us.
 // Layout: weights with a row stride of 65 words (rows and columns are both read
 // by 32 lanes without bank conflicts); activations as [feature][kTile], 12 words
 // apart (eight consecutive features' float4 fall into different banks).
-constexpr int kGradThreads = 128;
+constexpr int kGradThreads = 256;
 constexpr int kTile = 8;    // samples of a tile
 constexpr int kWLd = kMaxH + 1;
 constexpr int kALd = kTile + 4;
 
 struct GradSmem {  // offsets in floats
-    int w1, w2, w3, b1, b2, b3, x, h1, h2, z, dh2, dh1, loss, total;
+    int w1, w2, w3, b1, b2, b3, x, h1, h2, z, dh2, dh1, loss, half, total;
 };
 __host__ __device__ inline GradSmem grad_smem(const MlpDims& d) {
     GradSmem m;
@@ -89,6 +90,7 @@ __host__ __device__ inline GradSmem grad_smem(const MlpDims& d) {
     m.dh2 = take(kMaxH * kALd);
     m.dh1 = take(kMaxH * kALd);
     m.loss = take(kTile);
+    m.half = take(kMaxH * kALd);  // column sums over the second half of the inputs
     m.total = at;
     return m;
 }
@@ -111,7 +113,7 @@ __device__ __forceinline__ void load_rows(float* dst, const float* __restrict__ 
 
 // acc[i] += sum_k W(k) * a[k][sg * 4 + i] over k < K; W(k) = w[k * step]
 __device__ __forceinline__ void dot4(float (&acc)[4], const float* w, int step, const float* a, int K) {
-#pragma unroll 16
+#pragma unroll 8
     for (int k = 0; k < K; ++k) {
         const float wk = w[k * step];
         const float4 v = *reinterpret_cast<const float4*>(a + k * kALd);
@@ -123,14 +125,14 @@ __device__ __forceinline__ void dot4(float (&acc)[4], const float* w, int step, 
 }
 
 // g[j][c] += sum over the tile's samples of a[row_j][s] * b[col_c][s], rows
-// rg + 16 j, columns cg + 8 c.
+// rg + 32 j, columns cg + 8 c.
 template <int NR>
 __device__ __forceinline__ void outer(float (&g)[NR][8], const float* a, const float* b, int rg, int cg) {
-#pragma unroll
+#pragma unroll 1  // 128 registers: two CTAs per SM
     for (int h = 0; h < kTile; h += 4) {
         float4 u[NR];
 #pragma unroll
-        for (int j = 0; j < NR; ++j) u[j] = *reinterpret_cast<const float4*>(a + (rg + 16 * j) * kALd + h);
+        for (int j = 0; j < NR; ++j) u[j] = *reinterpret_cast<const float4*>(a + (rg + 32 * j) * kALd + h);
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             const float4 v = *reinterpret_cast<const float4*>(b + (cg + 8 * c) * kALd + h);
@@ -148,14 +150,14 @@ template <int NR>
 __device__ __forceinline__ void store_grad(float* out, const float (&g)[NR][8], int rows, int cols, int rg, int cg) {
 #pragma unroll
     for (int j = 0; j < NR; ++j) {
-        const int r = rg + 16 * j;
+        const int r = rg + 32 * j;
 #pragma unroll
         for (int c = 0; c < 8; ++c)
             if (r < rows && cg + 8 * c < cols) out[r * cols + cg + 8 * c] = g[j][c];
     }
 }
 
-__global__ void __launch_bounds__(kGradThreads) mlp_grad_kernel(MlpDims d, const float* __restrict__ params,
+__global__ void __launch_bounds__(kGradThreads, 2) mlp_grad_kernel(MlpDims d, const float* __restrict__ params,
                                                                 const float* __restrict__ X,
                                                                 const float* __restrict__ Q, int B,
                                                                 float* __restrict__ partial,
@@ -163,8 +165,8 @@ __global__ void __launch_bounds__(kGradThreads) mlp_grad_kernel(MlpDims d, const
     extern __shared__ __align__(16) float sm[];
     const GradSmem m = grad_smem(d);
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int col = t & 63, sg = t >> 6;      // forward and backward: a column, four samples
-    const int rg = t >> 3, cg = t & 7;        // weight gradients: rows rg + 16 j, columns cg + 8 c
+    const int col = t & 63, sg = (t >> 6) & 1, kh = t >> 7;  // a column, four samples, half of the inputs
+    const int rg = t >> 3, cg = t & 7;                       // weight gradients: rows rg + 32 j, columns cg + 8 c
     grid_dependency_wait();  // the step before may have just written the parameters
     allow_dependents();
     load_rows(sm + m.w1, params + d.oW1, d.in, d.h);
@@ -177,7 +179,7 @@ __global__ void __launch_bounds__(kGradThreads) mlp_grad_kernel(MlpDims d, const
     }
     // rows past the network's own sizes are read by the outer products: zero them once
     for (int i = t; i < m.loss - m.x; i += kGradThreads) sm[m.x + i] = 0.f;
-    float g1[2][8] = {}, g2[4][8] = {}, g3[4][8] = {};  // W1 (in <= 32), W2, W3
+    float g1[1][8] = {}, g2[2][8] = {}, g3[2][8] = {};  // W1 (in <= 32), W2, W3
     float gb[3] = {};                                   // thread t < 64: entry t of b1, b2, b3
     float loss = 0.f;                                   // thread 0
     const float invB = 1.0f / (float)B;
@@ -189,41 +191,56 @@ __global__ void __launch_bounds__(kGradThreads) mlp_grad_kernel(MlpDims d, const
             const int s = i / d.in, f = i - s * d.in;
             sm[m.x + f * kALd + s] = s < nb ? X[(int64_t)b0 * d.in + i] : 0.f;
         }
-        float q[2][2];  // this warp's two samples' targets, for the softmax below
+        float q[2];  // this warp's sample's targets, for the softmax below
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int s = 2 * warp + k;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int o = lane + 32 * h;
-                q[k][h] = (s < nb && o < d.out) ? Q[(int64_t)(b0 + s) * d.out + o] : 0.f;
-            }
+        for (int h = 0; h < 2; ++h) {
+            const int o = lane + 32 * h;
+            q[h] = (warp < nb && o < d.out) ? Q[(int64_t)(b0 + warp) * d.out + o] : 0.f;
         }
         asm volatile("cp.async.wait_all;" ::: "memory");  // the first tile: the weights
         __syncthreads();
-        // one layer's column `col` for samples 4 sg .. 4 sg + 3; samples past the batch are zero
-        auto layer = [&](int w, int bias, int src, int K, int dst, bool relu) {
-            const float bv = sm[bias + col];
-            float a[4] = {bv, bv, bv, bv};
-            dot4(a, sm + w + col, kWLd, sm + src + sg * 4, K);
-            float4 r;
-            float* rv = reinterpret_cast<float*>(&r);
+        // a column's sum over K inputs for samples 4 sg .. 4 sg + 3, from `init`: each half
+        // of the threads takes half of the inputs, the second leaves its sum in `half`
+        float* half = sm + m.half + col * kALd + sg * 4;
+        auto half_dot = [&](float (&a)[4], const float* w, int step, const float* src, int K, float init) {
+            const int k0 = (K + 1) / 2;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) rv[i] = (sg * 4 + i < nb && !(relu && !(a[i] > 0.f))) ? a[i] : 0.f;
-            *reinterpret_cast<float4*>(sm + dst + col * kALd + sg * 4) = r;
+            for (int i = 0; i < 4; ++i) a[i] = kh == 0 ? init : 0.f;
+            if (kh == 0) dot4(a, w, step, src + sg * 4, k0);
+            else dot4(a, w + k0 * step, step, src + k0 * kALd + sg * 4, K - k0);
+            if (kh == 1) *reinterpret_cast<float4*>(half) = make_float4(a[0], a[1], a[2], a[3]);
+        };
+        auto add_half = [&](float (&a)[4]) {
+            const float4 v = *reinterpret_cast<const float4*>(half);
+            a[0] += v.x;
+            a[1] += v.y;
+            a[2] += v.z;
+            a[3] += v.w;
+        };
+        // one layer; samples past the batch are zero
+        auto layer = [&](int w, int bias, int src, int K, int dst, bool relu) {
+            float a[4];
+            half_dot(a, sm + w + col, kWLd, sm + src, K, sm[bias + col]);
+            __syncthreads();
+            if (kh == 0) {
+                add_half(a);
+                float4 r;
+                float* rv = reinterpret_cast<float*>(&r);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) rv[i] = (sg * 4 + i < nb && !(relu && !(a[i] > 0.f))) ? a[i] : 0.f;
+                *reinterpret_cast<float4*>(sm + dst + col * kALd + sg * 4) = r;
+            }
             __syncthreads();
         };
         layer(m.w1, m.b1, m.x, d.in, m.h1, true);
         layer(m.w2, m.b2, m.h1, d.h, m.h2, true);
         layer(m.w3, m.b3, m.h2, d.h, m.z, false);
-        // softmax cross-entropy, two samples per warp: z becomes (p - q) / B
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int s = 2 * warp + k;
+        // softmax cross-entropy, one sample per warp: z becomes (p - q) / B
+        {
             float z[2], mx = -INFINITY;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                z[h] = lane + 32 * h < d.out ? sm[m.z + (lane + 32 * h) * kALd + s] : -INFINITY;
+                z[h] = lane + 32 * h < d.out ? sm[m.z + (lane + 32 * h) * kALd + warp] : -INFINITY;
                 mx = fmaxf(mx, z[h]);
             }
             for (int off = 16; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
@@ -237,24 +254,30 @@ __global__ void __launch_bounds__(kGradThreads) mlp_grad_kernel(MlpDims d, const
             for (int h = 0; h < 2; ++h) {
                 const int o = lane + 32 * h;
                 if (o < d.out) {
-                    sm[m.z + o * kALd + s] = s < nb ? (expf(z[h] - lse) - q[k][h]) * invB : 0.f;
-                    l += q[k][h] * (lse - z[h]);
+                    sm[m.z + o * kALd + warp] = warp < nb ? (expf(z[h] - lse) - q[h]) * invB : 0.f;
+                    l += q[h] * (lse - z[h]);
                 }
             }
             for (int off = 16; off; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
-            if (lane == 0) sm[m.loss + s] = s < nb ? l * invB : 0.f;
+            if (lane == 0) sm[m.loss + warp] = warp < nb ? l * invB : 0.f;
         }
         __syncthreads();
-        // backward: row `col` of W for the tile's samples, masked by the activation's sign
-        auto back = [&](int w, int src, int K, int act, int dst) {
-            if (col < d.h) {
-                float a[4] = {0.f, 0.f, 0.f, 0.f};
-                dot4(a, sm + w + col * kWLd, 1, sm + src + sg * 4, K);
+        // backward: row `col` of W for the tile's samples, masked by the activation's
+        // sign, in two steps around the barrier that the outer product before it shares
+        float a[4];
+        auto back = [&](int w, int src, int K) {
+            if (col < d.h) half_dot(a, sm + w + col * kWLd, 1, sm + src, K, 0.f);
+        };
+        auto back_end = [&](int act, int dst) {
+            __syncthreads();
+            if (kh == 0 && col < d.h) {
+                add_half(a);
                 const float4 h = *reinterpret_cast<const float4*>(sm + act + col * kALd + sg * 4);
                 *reinterpret_cast<float4*>(sm + dst + col * kALd + sg * 4) =
                     make_float4(h.x > 0.f ? a[0] : 0.f, h.y > 0.f ? a[1] : 0.f, h.z > 0.f ? a[2] : 0.f,
                                 h.w > 0.f ? a[3] : 0.f);
             }
+            __syncthreads();
         };
         auto bias_grad = [&](float& g, int src) {
             if (t < kMaxH) {
@@ -262,18 +285,18 @@ __global__ void __launch_bounds__(kGradThreads) mlp_grad_kernel(MlpDims d, const
                 for (int s = 0; s < kTile; ++s) g += sm[src + t * kALd + s];
             }
         };
-        back(m.w3, m.z, d.out, m.h2, m.dh2);
+        back(m.w3, m.z, d.out);
         outer(g3, sm + m.h2, sm + m.z, rg, cg);
         bias_grad(gb[2], m.z);
         if (t == 0) {
 #pragma unroll
             for (int s = 0; s < kTile; ++s) loss += sm[m.loss + s];
         }
-        __syncthreads();
-        back(m.w2, m.dh2, d.h, m.h1, m.dh1);
+        back_end(m.h2, m.dh2);
+        back(m.w2, m.dh2, d.h);
         outer(g2, sm + m.h1, sm + m.dh2, rg, cg);
         bias_grad(gb[1], m.dh2);
-        __syncthreads();
+        back_end(m.h1, m.dh1);
         outer(g1, sm + m.x, sm + m.dh1, rg, cg);
         bias_grad(gb[0], m.dh1);
         __syncthreads();
