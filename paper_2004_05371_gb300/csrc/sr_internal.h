@@ -68,6 +68,7 @@ struct SegPlan {
     int stage = 0;
     bool comp = false, fp64 = false, dense = false, bulk = false, warp = false, lane = false, adapt = false;
     int vec = 16, unroll = 4, block = 256, grid = 0;
+    int cta = 0;      // threads of the CTAs launched (block, but for the adaptive form's nominal one)
     int stages = 0;
     int ring = 0;     // TMA form: stages the kernel runs with (see plan_tma)
     size_t smem = 0;  // dynamic shared memory of the TMA form

@@ -37,6 +37,7 @@ constexpr int kSegFormFlags =
 // atomically.  2^21 segments of 16: 61.8 us with the 16 MiB zeroed, 54.6 with
 // tickets; 90,000 of 16: 9.6 against 11.7.
 constexpr int64_t kSegZeroMax = 1 << 19;
+constexpr int kTmaBlock = 384;          // TMA form: threads of a CTA when no part of the shape is given
 constexpr int kAdaptMaxCtasPerSm = 4;  // adaptive form: largest grid it takes, in CTAs per SM
 constexpr int64_t kSegAdaptMin = 4096;  // segments from which the default is the adaptive form
 constexpr int64_t kSegBulkMin = 32768;  // segments from which the default shape is the TMA form
@@ -65,7 +66,7 @@ bool seg_kernels(int dtype, bool comp, int vec, int unroll, bool dense, bool war
     return *main != nullptr;
 }
 
-// The TMA form's kernel for p (block and stages set) with chunks of `unroll`
+// The TMA form's kernel for p (cta and stages set) with chunks of `unroll`
 // rows of 32 `vec`-byte vectors; its second kernel, shared memory (per warp:
 // stages of a chunk and an mbarrier each, and the strip table) and resident CTAs.
 int plan_tma(SegPlan& p, int vec, int unroll, const DeviceInfo& d, int* resident) {
@@ -76,19 +77,19 @@ int plan_tma(SegPlan& p, int vec, int unroll, const DeviceInfo& d, int* resident
     default: p.main = seg_tma_fp8(p.comp, vec, unroll); seg_ldg_fp8(p.comp, vec, unroll, &p.fin); break;
     }
     if (!p.main) return SR_ERR_UNSUPPORTED;
-    const size_t ring = (size_t)(p.block / 32) * p.stages * ((size_t)unroll * 32 * vec + 8);
+    const size_t ring = (size_t)(p.cta / 32) * p.stages * ((size_t)unroll * 32 * vec + 8);
     p.ring = p.stages;
-    p.smem = ring + (size_t)(p.block / 32) * kStripTableBytes;
+    p.smem = ring + (size_t)(p.cta / 32) * kStripTableBytes;
     if (p.smem > (size_t)d.smem_per_block_optin) return SR_ERR_LAUNCH;
     int st = prepare_function(p.main, p.smem, false);
     if (st != SR_OK) return st;
-    st = blocks_per_sm(d, p.main, p.block, p.smem, resident);
+    st = blocks_per_sm(d, p.main, p.cta, p.smem, resident);
     if (st != SR_OK) return st;
     if (p.stages > 2) {
         // a few shapes fill the SM so closely that the tables would cost a CTA:
         // they take the place of one stage there
         int bare = 0;
-        st = blocks_per_sm(d, p.main, p.block, ring, &bare);
+        st = blocks_per_sm(d, p.main, p.cta, ring, &bare);
         if (st != SR_OK) return st;
         if (bare > *resident) {
             *resident = bare;
@@ -184,6 +185,7 @@ int seg_plan(int64_t nseg, int dtype, const sr_config& c, const DeviceInfo& d, S
         if (c.grid > (int64_t)kAdaptMaxCtasPerSm * d.sms) return SR_ERR_LAUNCH;
         p.stage = SR_LAST_BLOCK;  // the stage bits are ignored
         p.block = 256;
+        p.cta = kTmaBlock;
         p.stages = 2;
         int resident = 0;
         int st = plan_tma(p, 32, 4, d, &resident);
@@ -191,8 +193,8 @@ int seg_plan(int64_t nseg, int dtype, const sr_config& c, const DeviceInfo& d, S
         p.vec = 16;
         p.unroll = 2;
         const int64_t grid = c.grid ? c.grid : (int64_t)resident * d.sms;
-        p.grid = (int)std::max<int64_t>(1, std::min<int64_t>(grid, kSegMaxWarps / (p.block / 32)));
-        p.warps = (int64_t)p.grid * (p.block / 32);
+        p.grid = (int)std::max<int64_t>(1, std::min<int64_t>(grid, kSegMaxWarps / (p.cta / 32)));
+        p.warps = (int64_t)p.grid * (p.cta / 32);
         *out = p;
         return SR_OK;
     }
@@ -206,6 +208,8 @@ int seg_plan(int64_t nseg, int dtype, const sr_config& c, const DeviceInfo& d, S
     // 10,000 it is 1-3 % behind.
     p.bulk = (c.variant & SR_F_BULK) != 0 || (!shape_given && !p.dense && !p.warp && !p.lane && nseg >= kSegBulkMin);
     int st, resident = 0;
+    if (p.bulk && !shape_given && !c.grid && !c.ctas_per_sm) p.block = kTmaBlock;
+    p.cta = p.block;
     if (p.bulk) {
         if (!c.unroll) p.unroll = 4;
         p.stages = c.stages ? c.stages : 2;
@@ -289,10 +293,10 @@ int seg_launch(const void* x, const int64_t* offsets, void* out, const SegPlan& 
     lc.attrs = pdl;
     lc.numAttrs = 1;
     if (p.stage == SR_GRID_SYNC && !p.warp && !p.lane) {
-        e = cudaLaunchCooperativeKernel(p.main, dim3(p.grid), dim3(p.block), args, p.smem, s);
+        e = cudaLaunchCooperativeKernel(p.main, dim3(p.grid), dim3(p.cta), args, p.smem, s);
     } else {
         lc.gridDim = dim3(p.grid);
-        lc.blockDim = dim3(p.block);
+        lc.blockDim = dim3(p.cta);
         lc.dynamicSmemBytes = p.smem;
         e = cudaLaunchKernelExC(&lc, p.main, args);
         lc.dynamicSmemBytes = 0;

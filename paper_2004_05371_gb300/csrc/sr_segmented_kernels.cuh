@@ -542,14 +542,15 @@ __global__ void __launch_bounds__(512, 1) seg_kernel(const SegParams p) {
 // BF16 values at 1.8 TB/s.  Now a chunk with ends in it costs about 450 warp
 // instructions whatever their number, where HBM leaves time for some 650.
 // Device time before and now (~2^28 elements unless said otherwise):
-//   f32   1M x 268             343 -> 178 us      f32  4M lognormal    1013 -> 200 us
-//   f32   4M x 64              915 -> 189         f32  16M x 16        3110 -> 229
-//   bf16  1M x 268 (0..536)    297 -> 102         fp8  100k lognormal   160 ->  63
-//   i32   2^21 x 16 (0..32)    525 ->  55         bf16 4M x 39, lognormal 868 -> 115
+//   f32   1M x 268             343 -> 177 us      f32  4M lognormal    1013 -> 191 us
+//   f32   4M x 64              915 -> 188         f32  16M x 16        3110 -> 209
+//   bf16  1M x 268 (0..536)    297 -> 100         fp8  100k lognormal   160 ->  61
+//   i32   2^21 x 16 (0..32)    525 ->  53         bf16 4M x 39, lognormal 868 -> 113
 // What bounds it now: instructions (55-70 % of the issue slots) from about five
-// ends per chunk up, HBM below.  80 registers, so three 256-thread CTAs (24 warps)
-// are resident with two 4 KiB stages each: 16 warps of 112 registers took 4 %
-// less on long segments and 8-12 % more on short ones.
+// ends per chunk up, HBM below, and 4-7 us of search and first copies at the start.
+// 80 registers, so 24 warps (two 384-thread CTAs, 1 % ahead of three of 256) are
+// resident with two 4 KiB stages each: 16 warps of 112 registers took 4 % less on
+// long segments and 8-12 % more on short ones.
 
 // Sum of the elements in one 16-byte vector (four 32-bit words); compensated
 // binary32 and BF16 go through PackedPairs (below) instead.
@@ -675,7 +676,10 @@ template <int EB> __device__ __forceinline__ void keep_from(uint32_t (&r)[4], in
     }
 }
 
-constexpr int kAheadOffsets = 256;   // offsets fetched into L2 this far ahead of the window
+// Offsets fetched into L2 this far ahead of the window: the one after `nxt`.  Further
+// ahead they are more often gone again (16M x 16 f32: 211 us with 64, 216 with 192,
+// 231 with 256).
+constexpr int kAheadOffsets = 64;
 // Longest segment (bytes) one lane sums alone, about where that costs a chunk
 // as many instructions as the strips do.
 template <int DT> struct OwnBytes { static constexpr int v = 256; };
