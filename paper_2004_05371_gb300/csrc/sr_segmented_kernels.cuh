@@ -199,40 +199,45 @@ template <class P> __device__ __forceinline__ P carry_load(const unsigned char* 
 
 // Finish a spanning segment s owned by warp w_o, ending in warp w_e (whole
 // warp calls; fixed order, so the result does not depend on which warp runs it).
-template <class P> __device__ __forceinline__ void finish_span_typed(const SegParams& p, int64_t s, int64_t w_o,
-                                                                     int64_t w_e, int lane) {
-    P first = Op<P>::zero(), acc = Op<P>::zero();
-    if (lane == 0) first = carry_load<P>(p.carry_last, w_o);
+// WIDE: eight loads in flight, for a long segment has thousands of carries (one of
+// 2^24 elements 22.2 -> 20.0 us).  The LDG kernel keeps the plain loop: with the
+// wide one its hot loop got fewer registers (10,000 lognormal segments at 32 B x 4:
+// 168 -> 205 us).
+template <class P, bool WIDE> __device__ __forceinline__ void finish_span_typed(const SegParams& p, int64_t s,
+                                                                                int64_t w_o, int64_t w_e, int lane) {
+    P acc = Op<P>::zero();
     int64_t w = w_o + 1 + lane;
-    for (; w + 7 * 32 <= w_e; w += 8 * 32) {  // eight loads in flight: a long segment has thousands of carries
-        P c[8];
+    if constexpr (WIDE) {
+        for (; w + 7 * 32 <= w_e; w += 8 * 32) {
+            P c[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) c[k] = carry_load<P>(p.carry_first, w + 32 * k);
+            for (int k = 0; k < 8; ++k) c[k] = carry_load<P>(p.carry_first, w + 32 * k);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) acc = Op<P>::add(acc, c[k]);
+            for (int k = 0; k < 8; ++k) acc = Op<P>::add(acc, c[k]);
+        }
     }
     for (; w <= w_e; w += 32) acc = Op<P>::add(acc, carry_load<P>(p.carry_first, w));
     acc = warp_reduce(acc);
     if (lane == 0) {
-        P total = Op<P>::add(first, acc);
+        P total = Op<P>::add(carry_load<P>(p.carry_last, w_o), acc);
         if constexpr (std::is_same<P, double>::value) seg_out_d(p, s, total);
         else seg_out(p, s, total);
     }
 }
-template <class A> __device__ __forceinline__ void finish_span(const SegParams& p, int64_t s, int64_t w_o,
-                                                               int64_t w_e, int lane) {
+template <class A, bool WIDE> __device__ __forceinline__ void finish_span(const SegParams& p, int64_t s, int64_t w_o,
+                                                                          int64_t w_e, int lane) {
     if constexpr (std::is_same<A, long long>::value) {
-        finish_span_typed<long long>(p, s, w_o, w_e, lane);
+        finish_span_typed<long long, WIDE>(p, s, w_o, w_e, lane);
     } else {
-        if (p.fp64) finish_span_typed<double>(p, s, w_o, w_e, lane);
-        else finish_span_typed<A>(p, s, w_o, w_e, lane);
+        if (p.fp64) finish_span_typed<double, WIDE>(p, s, w_o, w_e, lane);
+        else finish_span_typed<A, WIDE>(p, s, w_o, w_e, lane);
     }
 }
 
 // Per-segment ticket of the last-block form: every contributing warp
 // arrives once; the last one finishes the segment and resets the ticket.
-template <class A> __device__ __forceinline__ void span_arrive(const SegParams& p, int64_t s, int64_t w_o,
-                                                               int64_t w_e, int lane) {
+template <class A, bool WIDE> __device__ __forceinline__ void span_arrive(const SegParams& p, int64_t s, int64_t w_o,
+                                                                          int64_t w_e, int lane) {
     unsigned t = 0;
     if (lane == 0) {
         __threadfence();
@@ -241,7 +246,7 @@ template <class A> __device__ __forceinline__ void span_arrive(const SegParams& 
     t = __shfl_sync(0xffffffffu, t, 0);
     if (t == (unsigned)(w_e - w_o)) {
         __threadfence();
-        finish_span<A>(p, s, w_o, w_e, lane);
+        finish_span<A, WIDE>(p, s, w_o, w_e, lane);
         if (lane == 0) atomicExch(p.cnt + w_o, 0u);
     }
 }
@@ -320,7 +325,7 @@ __global__ void __launch_bounds__(512, 1) seg_kernel(const SegParams p) {
             } else {
                 if (lane == 0) carry_store(p, p.carry_first, w, v);
                 if (p.stage == kStageLastBlock)
-                    span_arrive<A>(p, s, (cur_start - base) / E, (cur_end - 1 - base) / E, lane);
+                    span_arrive<A, false>(p, s, (cur_start - base) / E, (cur_end - 1 - base) / E, lane);
             }
         } else if (cur_end <= hi) {  // owned and complete
             if (lane == 0) seg_out(p, s, v);
@@ -330,7 +335,7 @@ __global__ void __launch_bounds__(512, 1) seg_kernel(const SegParams p) {
                 if (lane == 0) seg_atomic(p, s, v);
             } else {
                 if (lane == 0) carry_store(p, p.carry_last, w, v);
-                if (p.stage == kStageLastBlock) span_arrive<A>(p, s, w, (cur_end - 1 - base) / E, lane);
+                if (p.stage == kStageLastBlock) span_arrive<A, false>(p, s, w, (cur_end - 1 - base) / E, lane);
             }
         }
         cur += 1;
@@ -512,7 +517,7 @@ __global__ void __launch_bounds__(512, 1) seg_kernel(const SegParams p) {
         g.sync();
         if (spanning >= 0) {
             const int64_t end = __ldg(p.offsets + spanning + 1);
-            finish_span<A>(p, spanning, w, (end - 1 - base) / E, lane);
+            finish_span<A, false>(p, spanning, w, (end - 1 - base) / E, lane);
         }
     }
 }
@@ -786,7 +791,7 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
         }
         if (lane == 0) carry_store(p, p.carry_first, w, v);
         if (p.stage == kStageLastBlock)
-            span_arrive<A>(p, s, (__ldg(p.offsets + s) - base) / E, (__ldg(p.offsets + s + 1) - 1 - base) / E, lane);
+            span_arrive<A, true>(p, s, (__ldg(p.offsets + s) - base) / E, (__ldg(p.offsets + s + 1) - 1 - base) / E, lane);
     };
     // the open segment's sum so far, in lane 0; acc restarts at zero
     auto take_acc = [&]() {
@@ -1103,7 +1108,7 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
             } else {
                 if (lane == 0) carry_store(p, p.carry_last, w, v);
                 if (p.stage == kStageLastBlock)
-                    span_arrive<A>(p, spanning, w, (cur_end - 1 - base) / E, lane);
+                    span_arrive<A, true>(p, spanning, w, (cur_end - 1 - base) / E, lane);
             }
             break;  // the next segment starts in the next warp's piece
         }
@@ -1121,7 +1126,7 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
         g.sync();
         if (spanning >= 0) {
             const int64_t end = __ldg(p.offsets + spanning + 1);
-            finish_span<A>(p, spanning, w, (end - 1 - base) / E, lane);
+            finish_span<A, true>(p, spanning, w, (end - 1 - base) / E, lane);
         }
     }
 }
@@ -1144,7 +1149,7 @@ __global__ void __launch_bounds__(256) seg_finish_kernel(const SegParams p, int6
     E = ((E + PV - 1) / PV) * PV;
     if (E < e_min) E = e_min;
     const int64_t end = __ldg(p.offsets + s + 1);
-    finish_span<A>(p, s, w, (end - 1 - base) / E, lane);
+    finish_span<A, true>(p, s, w, (end - 1 - base) / E, lane);
 }
 
 // The dense variant exists for at most 4 rows in flight per warp: with 8 its
