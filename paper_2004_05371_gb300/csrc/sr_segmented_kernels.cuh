@@ -835,17 +835,27 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
         const uint32_t va = (unsigned)a / EV, vb = (unsigned)(b - 1) / EV;
         const int nb = b - (int)vb * EV;  // elements of the last vector
         uint32_t r[4];
-        if constexpr (kCompact) {
-            uint32_t i = va + ((uint32_t)lane & 7u);
-            if (i > vb) i = va;
+        if constexpr (DT == kDtFP8) {
+            // one copy of the code: the first vector, the last, then those between, so
+            // that all lanes mask in the same two steps (masked wherever a lane's turn
+            // came, nearly every step did: 1.5M segments of 41 49.2 -> 46.4 us, 4M of 64 78.8 -> 74.2)
+            uint32_t i = va, next = va + 1u + ((uint32_t)lane & 7u);
+            if (next >= vb) next = va + 1u;
             VP v = VP::zero();
 #pragma unroll 1
-            for (uint32_t k = va; k <= vb; ++k) {
+            for (uint32_t k = 0; k <= vb - va; ++k) {
                 lds_vec(sb + 16u * i, r);
-                if (i == va) keep_from<EB>(r, a & (EV - 1));
-                if (i == vb) keep_below<EB>(r, nb);
+                if (k < 2) {
+                    if (k == 0) keep_from<EB>(r, a & (EV - 1));
+                    if (i == vb) keep_below<EB>(r, nb);
+                }
                 v.add(VP::of(r));
-                if (++i > vb) i = va;
+                if (k == 0) {
+                    i = vb;
+                } else {
+                    i = next;
+                    if (++next >= vb) next = va + 1u;
+                }
             }
             return v.total();
         } else {  // the masked ends apart from the whole vectors between them
@@ -919,7 +929,7 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
             const int np = ahead < ce ? (int)ahead : 2 * CE;
             int npp = __shfl_up_sync(0xffffffffu, np, 1);
             if (lane == 0) npp = last;
-                short_only = !__any_sync(0xffffffffu, np < ce && np - npp > kOwn);
+            short_only = !__any_sync(0xffffffffu, np < ce && np - npp > kOwn);
         }
         while (short_only) {
             const int from = rpp > 0 ? rpp : 0;
