@@ -197,26 +197,54 @@ template <class P> __device__ __forceinline__ P carry_load(const unsigned char* 
     }
 }
 
+// A running sum of partial sums whose number grows with the input.  A plain
+// binary32 chain of k same-sign additions errs by up to k u |S| (64 additions of
+// 0.1f exceed 4 eps32 |S|), so there it carries the rounding errors along
+// (TwoSum); int64 is exact, pairs carry theirs already, and binary64 has room.
+template <class A> struct RunSum {
+    A v;
+    __device__ __forceinline__ static RunSum of(A x) { return RunSum{x}; }
+    __device__ __forceinline__ void add(A x) { v = Op<A>::add(v, x); }
+    __device__ __forceinline__ A total() const { return v; }
+    __device__ __forceinline__ A only() const { return v; }  // the sum when nothing was added to it
+};
+template <> struct RunSum<float> {
+    float s, c;
+    __device__ __forceinline__ static RunSum of(float x) { return RunSum{x, 0.f}; }
+    __device__ __forceinline__ void add(float x) {
+        float t, e;
+        two_sum(s, x, t, e);
+        s = t;
+        c = __fadd_rn(c, e);
+    }
+    // an infinite sum leaves a NaN correction
+    __device__ __forceinline__ float total() const { return c == c ? __fadd_rn(s, c) : s; }
+    __device__ __forceinline__ float only() const { return s; }
+};
+
 // Finish a spanning segment s owned by warp w_o, ending in warp w_e (whole
 // warp calls; fixed order, so the result does not depend on which warp runs it).
 // WIDE: eight loads in flight, for a long segment has thousands of carries (one of
-// 2^24 elements 22.2 -> 20.0 us).  The LDG kernel keeps the plain loop: with the
-// wide one its hot loop got fewer registers (10,000 lognormal segments at 32 B x 4:
-// 168 -> 205 us).
+// 2^24 elements 22.2 -> 20.0 us), added as a tree and those trees' sums as a RunSum.
+// The LDG kernel keeps the plain loop: with the wide one its hot loop got fewer
+// registers (10,000 lognormal segments at 32 B x 4: 168 -> 205 us).
 template <class P, bool WIDE> __device__ __forceinline__ void finish_span_typed(const SegParams& p, int64_t s,
                                                                                 int64_t w_o, int64_t w_e, int lane) {
     P acc = Op<P>::zero();
     int64_t w = w_o + 1 + lane;
     if constexpr (WIDE) {
+        RunSum<P> sum = RunSum<P>::of(acc);
         for (; w + 7 * 32 <= w_e; w += 8 * 32) {
             P c[8];
 #pragma unroll
             for (int k = 0; k < 8; ++k) c[k] = carry_load<P>(p.carry_first, w + 32 * k);
-#pragma unroll
-            for (int k = 0; k < 8; ++k) acc = Op<P>::add(acc, c[k]);
+            sum.add(sum_words<P, 8>(c));
         }
+        for (; w <= w_e; w += 32) sum.add(carry_load<P>(p.carry_first, w));
+        acc = sum.total();
+    } else {
+        for (; w <= w_e; w += 32) acc = Op<P>::add(acc, carry_load<P>(p.carry_first, w));
     }
-    for (; w <= w_e; w += 32) acc = Op<P>::add(acc, carry_load<P>(p.carry_first, w));
     acc = warp_reduce(acc);
     if (lane == 0) {
         P total = Op<P>::add(carry_load<P>(p.carry_last, w_o), acc);
@@ -771,8 +799,11 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
     if (cont) cur_start = lo;
     int kb = cont ? r0 : r0 + 1;
     int64_t cur_end = __shfl_sync(0xffffffffu, win, kb);
-    A acc = Op<A>::zero();  // this lane's part of the open segment
-    bool spread = false;    // acc is nonzero in lanes other than lane 0
+    // This lane's part of the open segment: one addition per chunk, 72 in a warp's piece
+    // of 2^28 binary32 elements (in a plain chain, constant data came out 5.6 eps32 off
+    // in 4200 segments of 60,000 where 4 is the gate).
+    RunSum<A> acc = RunSum<A>::of(Op<A>::zero());
+    bool spread = false;  // acc is nonzero in lanes other than lane 0
 
     auto next_window = [&]() {
         win = nxt;
@@ -795,8 +826,8 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
     };
     // the open segment's sum so far, in lane 0; acc restarts at zero
     auto take_acc = [&]() {
-        const A v = spread ? warp_reduce(acc) : acc;
-        acc = Op<A>::zero();
+        const A v = spread ? warp_reduce(acc.total()) : acc.only();
+        acc = RunSum<A>::of(Op<A>::zero());
         spread = false;
         return v;
     };
@@ -816,7 +847,7 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
         A one = Op<A>::zero();
         if (idx < b1) acc_elem<DT>(one, p.x, idx);
         for (;;) {
-            if (idx < b1 && idx >= cur_start && idx < cur_end) acc = Op<A>::add(acc, one);
+            if (idx < b1 && idx >= cur_start && idx < cur_end) acc.add(one);
             if (cur_end > b0) spread = true;
             if (cur_end >= b1) break;
             emit_advance();
@@ -895,7 +926,7 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
                 v[1].add(VP::of(r1));
             }
             v[0].add(v[1]);
-            acc = Op<A>::add(acc, v[0].total());
+            acc.add(v[0].total());
             spread = true;
             return;
         }
@@ -958,7 +989,7 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
                 if (k == (unsigned)prev / EV) keep_from<EB>(r, prev & (EV - 1));
                 t.add(VP::of(r));
             }
-            acc = t.total();
+            acc = RunSum<A>::of(t.total());
             spread = true;
             cur_start = c0 + prev;
             cur_end = __shfl_sync(0xffffffffu, win, kb);
@@ -1028,10 +1059,7 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
             keep_from<EB>(r, ql & (EV - 1));
             tv.add(VP::of(r));
         }
-        // the open segment of the chunks before enters at strip 0
-        A head = hv.total();
-        const A before = take_acc();
-        if (lane == 0) head = Op<A>::add(before, head);
+        const A head = hv.total();
         // segmented inclusive scan of the open runs over the strips: before the
         // step with distance d a lane's partial covers lanes [lane - d + 1,
         // lane], and takes in the lanes before them unless one of its own holds
@@ -1047,9 +1075,13 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
         A closed = Op<A>::shfl_up(x, 1);  // the run open at the end of the strip before
         closed = lane == 0 ? head : Op<A>::add(closed, head);
         const A open_end = Op<A>::shfl(x, 31);
-        if (lane == 0) acc = open_end;
-        if (cont) {  // the first segment to end began in an earlier warp's piece
-            const int fl = __ffs(tmask) - 1;
+        // the open segment of the chunks before is the first to end: its sum is rounded
+        // once here (entering at strip 0 it was rounded at every step of the scan)
+        const int fl = __ffs(tmask) - 1;
+        const A before = Op<A>::shfl(take_acc(), 0);
+        if (lane == fl) closed = Op<A>::add(before, closed);
+        if (lane == 0) acc = RunSum<A>::of(open_end);
+        if (cont) {  // it began in an earlier warp's piece
             emit_first(__shfl_sync(0xffffffffu, qseg, fl), Op<A>::shfl(closed, fl));
             closes = closes && lane != fl;
         }
