@@ -720,6 +720,97 @@ template <> struct OwnBytes<kDtI32> { static constexpr int v = 192; };
 template <> struct OwnBytes<kDtBF16> { static constexpr int v = 192; };
 template <> struct OwnBytes<kDtFP8> { static constexpr int v = 128; };
 
+// Runs of empty segments (padded offsets, keys that never occur) lie at one element, so the
+// split by elements leaves a whole run to one warp: a million segments of 16 with three
+// million empty ones behind them took 560 ms, one step each.  Now (32 us without the run):
+// 36 us with it behind or before the data, 41 in the middle.
+//   - The blocks of kEmptyBlock segments that are all empty are zeroed by all warps in turn
+//     (two loads per block, beside the kernel's first ones).
+//   - The warp that comes upon a run where a chunk or the piece starts or ends looks for the
+//     run's end and writes what lies outside those blocks (skip_empty).
+//   - A chunk takes the ends inside it a window of 32 at a time, 0.4 us each.  A piece with
+//     more than kFewSegments + 1/16 of its elements is therefore searched for runs of kRun
+//     entries and walked in stretches that end at them (next_run).  Fewer cost less than
+//     the looking: with 1/32, 16M segments of 16 lost another 1.5 %.
+// To look at every window instead costs 5-10 % on short segments: 4 instructions, but 60
+// more a chunk for registers that the strips then lack.
+constexpr int kEmptyBlock = 1024, kFewSegments = 1024, kRun = 512;
+
+// Zero out[a], ..., out[b - 1], `es` bytes each (4 or 8); whole warp calls.
+__device__ __forceinline__ void zero_out(void* out, int es, int64_t a, int64_t b, int lane) {
+    uint32_t* o = reinterpret_cast<uint32_t*>(out);
+    const int64_t hi = b * (es / 4);
+    for (int64_t i = a * (es / 4) + lane; i < hi; i += 32) o[i] = 0u;
+}
+// The window of offsets a warp of the strip kernel walks: lane k holds offsets[wb + k]
+// in win and offsets[wb + 32 + k] in nxt (INT64_MAX past the last).
+struct SegWindow {
+    int64_t wb, win, nxt;
+    int kb;  // entry of the open segment's end
+};
+__device__ __forceinline__ int64_t offset_at(const int64_t* off, int64_t nseg, int64_t i) {
+    return i <= nseg ? __ldg(off + i) : INT64_MAX;
+}
+
+// Closes the empty segments at element `at`, where the open segment starts (beyond two
+// windows, only those outside the blocks that are all empty), and opens the one after them.
+// Whole warp calls; out of line, or its registers would be taken from the strips (inlined:
+// 16M x 16 2-5 % slower).
+static __device__ __noinline__ SegWindow skip_empty(const int64_t* off, int64_t nseg, void* out, int es, int64_t at,
+                                                    SegWindow w) {
+    const int lane = threadIdx.x & 31;
+    for (;;) {
+        const int cnt = __popc(__ballot_sync(0xffffffffu, lane >= w.kb && w.win == at));
+        zero_out(out, es, w.wb + w.kb - 1, w.wb + w.kb - 1 + cnt, lane);
+        w.kb += cnt;
+        if (w.kb < 32) return w;
+        if (!__all_sync(0xffffffffu, w.nxt == at)) {
+            w.win = w.nxt;
+            w.wb += 32;
+        } else {
+            // lo: the first index with offsets[lo] > at (nseg + 1: none), looked for at
+            // power-of-two distances, then in 32 equal parts at a time
+            int64_t lo = w.wb + 64, hi = nseg + 1;
+            {
+                const int64_t k = lo + ((int64_t)1 << lane) - 1;
+                const unsigned m = __ballot_sync(0xffffffffu, k >= hi || __ldg(off + k) > at);
+                const int b = m ? __ffs(m) - 1 : 32;
+                if (b < 32) hi = min(hi, lo + ((int64_t)1 << b) - 1);
+                if (b > 0) lo += (int64_t)1 << (b - 1);
+            }
+            while (lo < hi) {
+                const int64_t step = (hi - lo + 31) / 32;
+                const int64_t k = lo + lane * step;
+                const unsigned m = __ballot_sync(0xffffffffu, k >= hi || __ldg(off + k) > at);
+                const int b = m ? __ffs(m) - 1 : 32;
+                if (b < 32) hi = min(hi, lo + b * step);
+                if (b > 0) lo += (b - 1) * step + 1;
+            }
+            // segments s0 .. end - 1 are empty too
+            const int64_t s0 = w.wb + 31, end = lo - 1;
+            const int64_t b0 = (s0 + kEmptyBlock - 1) / kEmptyBlock * kEmptyBlock, b1 = end / kEmptyBlock * kEmptyBlock;
+            zero_out(out, es, s0, min(end, b0), lane);
+            zero_out(out, es, max(b0, b1), end, lane);
+            w.wb = lo;
+            w.win = offset_at(off, nseg, lo + lane);
+        }
+        w.kb = 0;
+        w.nxt = offset_at(off, nseg, w.wb + 32 + lane);
+    }
+}
+
+// The element at which the first run of empty segments that takes kRun entries from entry i
+// of the offsets on (i + k kRun to i + k kRun + kRun) starts, before element `hi`; hi if
+// there is none (whole warp calls).
+static __device__ __noinline__ int64_t next_run(const int64_t* off, int64_t nseg, int64_t i, int64_t hi) {
+    const int lane = threadIdx.x & 31;
+    for (;; i += 32 * kRun) {
+        const int64_t a = offset_at(off, nseg, i + kRun * lane), b = offset_at(off, nseg, i + kRun * (lane + 1));
+        const unsigned m = __ballot_sync(0xffffffffu, a == b || b >= hi);
+        if (m != 0u) return min(hi, __shfl_sync(0xffffffffu, a == b ? a : hi, __ffs(m) - 1));
+    }
+}
+
 template <int DT, bool COMP, int VB, int UNROLL>
 __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
     using A = typename Acc<DT, COMP>::T;
@@ -741,8 +832,8 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
     allow_dependents();
     if (p.bad != nullptr && __ldcg(p.bad) != 0) return;  // offsets failed the check: read nothing
     const int lane = threadIdx.x & 31;
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t Wn = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int w = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // at most 65536 warps
+    const int Wn = (int)(gridDim.x * blockDim.x) >> 5;
     const int64_t base = __ldg(p.offsets);
     const int64_t N = __ldg(p.offsets + p.nseg) - base;
     int64_t E = (N + Wn - 1) / Wn;
@@ -751,14 +842,29 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
     const int64_t lo = base + (w * E < N ? w * E : N);
     const int64_t hi = base + ((w + 1) * E < N ? (w + 1) * E : N);
 
-    // geometry of the piece: scalar head [lo, c0), vector body of nch chunks
-    // (last_ce elements in the last), scalar tail [.., hi)
-    const uintptr_t addr = reinterpret_cast<uintptr_t>(p.x) + (uintptr_t)lo * EB;
-    int64_t c0 = lo + (int64_t)(((uintptr_t)VB - addr % VB) % VB) / EB;
-    if (c0 > hi) c0 = hi;
-    const int64_t body = (hi - c0) / PV * PV;
-    const int nch = (int)((body + CE - 1) / CE);
-    const int last_ce = (int)(body - (int64_t)(nch - 1) * CE);
+    // A stretch [from, to) of the piece (all of it, unless there are long runs of empty
+    // segments): scalar head, vector body of `left` chunks (last_ce elements in the last),
+    // scalar tail.
+    int head, left, last_ce, tail;
+    auto geometry = [&](int64_t from, int64_t to) {
+        const uintptr_t addr = reinterpret_cast<uintptr_t>(p.x) + (uintptr_t)from * EB;
+        head = (int)(((uintptr_t)VB - addr % VB) % VB) / EB;
+        if (head > to - from) head = (int)(to - from);
+        const int64_t body = (to - from - head) / PV * PV;
+        left = (int)((body + CE - 1) / CE);
+        last_ce = (int)(body - (int64_t)(left - 1) * CE);
+        tail = (int)(to - from - head - body);
+    };
+    geometry(lo, hi);
+    // segments that start at hi are this warp's too (elsewhere they are the next one's)
+    const bool last = w == Wn - 1 || base + (w + 1) * E > hi;
+    // base, E and hi are wanted only where a segment crosses the piece's ends or a stretch
+    // ends: the lanes keep a word each of them
+    const uint32_t stash = (uint32_t)((lane & 4 ? hi : lane & 2 ? E : base) >> (lane & 1 ? 32 : 0));
+    auto stashed = [&](int at) {
+        return (int64_t)((uint64_t)__shfl_sync(0xffffffffu, stash, at) |
+                         (uint64_t)__shfl_sync(0xffffffffu, stash, at + 1) << 32);
+    };
 
     extern __shared__ __align__(1024) unsigned char seg_dsm[];
     const int wib = threadIdx.x >> 5, nwib = blockDim.x >> 5, S = p.stages;
@@ -767,36 +873,43 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
     // the strip table: word t describes strip t's boundaries of one offsets window
     const uint32_t table =
         smem_u32(seg_dsm) + (uint32_t)(nwib * S) * (CHUNK + 8u) + (uint32_t)(wib * kStripTableBytes);
-    // lane 0: copy chunk k of the body into ring stage st, if there is one
-    auto issue = [&](const unsigned char* src, int k, int st) {
-        if (k >= nch) return;
-        const uint32_t bytes = k == nch - 1 ? (uint32_t)last_ce * EB : CHUNK;
+    // lane 0: copy the chunk at src, of l up to the last one, into ring stage st, if there is one
+    auto issue = [&](const unsigned char* src, int l, int st) {
+        if (l <= 0) return;
+        const uint32_t bytes = l == 1 ? (uint32_t)last_ce * EB : CHUNK;
         mbar_arrive_expect_tx(bars + 8u * st, bytes);
         bulk_g2s(ring + (uint32_t)st * CHUNK, src, bytes, bars + 8u * st);
     };
     // the ring's first copies (24 warps' rings are 30 MB for the chip: issued before
     // the search they held the searching warps up to 8 us, now 4)
+    int64_t wb, win, far;
     auto fill = [&]() {
+        far = offset_at(p.offsets, p.nseg, wb + kFewSegments + E / 16);
         if (lane == 0) {
-            for (int st = 0; st < S; ++st) mbar_init(bars + 8u * st, 1);
+            for (int j = 0; j < S; ++j) mbar_init(bars + 8u * j, 1);
             mbar_fence_init();
-            for (int st = 0; st < S; ++st) issue(p.x + (c0 + (int64_t)st * CE) * EB, st, st);
+            for (int j = 0; j < S; ++j) issue(p.x + (lo + head + (int64_t)j * CE) * EB, left - j, j);
         }
         __syncwarp();
     };
 
+    // this lane's block of segments, all empty if its first and last offset are equal
+    const int64_t nblk = p.nseg / kEmptyBlock;
+    int64_t blk = w + (int64_t)lane * Wn, blk0 = 0, blk1 = 1;
+    if (blk < nblk) {
+        blk0 = __ldg(p.offsets + blk * kEmptyBlock);
+        blk1 = __ldg(p.offsets + (blk + 1) * kEmptyBlock);
+    }
+
     // Stream state (warp-uniform).  The offsets window: lane k holds
     // offsets[wb + k] in win and offsets[wb + 32 + k] in nxt (loaded one window
     // ahead).  Entry kb is the end of the open segment, wb + kb - 1.
-    int64_t wb, win;
     const int64_t at = N > 0 ? (int64_t)((float)(w * E) / (float)N * (float)p.nseg) : 0;
     const int r0 =
         (int)(warp_search(p.offsets, p.nseg, base + w * E, at < p.nseg ? at : p.nseg, lane, wb, win, fill) - wb);
     int64_t nxt = (wb + 32 + lane <= p.nseg) ? __ldg(p.offsets + wb + 32 + lane) : INT64_MAX;
-    int64_t cur_start = __shfl_sync(0xffffffffu, win, r0);
-    // the open segment began in an earlier warp's piece (its true start is not needed)
-    bool cont = lo < hi && cur_start > lo;
-    if (cont) cur_start = lo;
+    // the open segment began in an earlier warp's piece
+    bool cont = lo < hi && __shfl_sync(0xffffffffu, win, r0) > lo;
     int kb = cont ? r0 : r0 + 1;
     int64_t cur_end = __shfl_sync(0xffffffffu, win, kb);
     // This lane's part of the open segment: one addition per chunk, 72 in a warp's piece
@@ -804,6 +917,19 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
     // in 4200 segments of 60,000 where 4 is the gate).
     RunSum<A> acc = RunSum<A>::of(Op<A>::zero());
     bool spread = false;  // acc is nonzero in lanes other than lane 0
+
+    for (;;) {  // blocks of empty segments
+        unsigned m = __ballot_sync(0xffffffffu, blk0 == blk1);
+        for (; m != 0u; m &= m - 1u) {
+            const int64_t b = __shfl_sync(0xffffffffu, blk, __ffs(m) - 1);
+            zero_out(p.out, std::is_same<A, long long>::value || p.fp64 ? 8 : 4, b * kEmptyBlock, (b + 1) * kEmptyBlock,
+                     lane);
+        }
+        blk += 32 * (int64_t)Wn;
+        if (__all_sync(0xffffffffu, blk >= nblk)) break;
+        blk0 = blk < nblk ? __ldg(p.offsets + blk * kEmptyBlock) : 0;
+        blk1 = blk < nblk ? __ldg(p.offsets + (blk + 1) * kEmptyBlock) : 1;
+    }
 
     auto next_window = [&]() {
         win = nxt;
@@ -821,8 +947,10 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
             return;
         }
         if (lane == 0) carry_store(p, p.carry_first, w, v);
-        if (p.stage == kStageLastBlock)
-            span_arrive<A, true>(p, s, (__ldg(p.offsets + s) - base) / E, (__ldg(p.offsets + s + 1) - 1 - base) / E, lane);
+        if (p.stage == kStageLastBlock) {
+            const int64_t b = stashed(0), e = stashed(2);
+            span_arrive<A, true>(p, s, (__ldg(p.offsets + s) - b) / e, (__ldg(p.offsets + s + 1) - 1 - b) / e, lane);
+        }
     };
     // the open segment's sum so far, in lane 0; acc restarts at zero
     auto take_acc = [&]() {
@@ -836,22 +964,16 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
         const A v = take_acc();
         if (cont) emit_first(wb + kb - 1, v);
         else if (lane == 0) seg_out(p, wb + kb - 1, v);
-        cur_start = cur_end;
         if (++kb == 32) next_window();
         cur_end = __shfl_sync(0xffffffffu, win, kb);
     };
-    // scalar chunk [b0, b1), at most 32 elements: lane l holds element b0 + l
-    auto scalar_chunk = [&](int64_t b0, int64_t b1) {
-        if (b0 >= b1) return;
-        const int64_t idx = b0 + lane;
-        A one = Op<A>::zero();
-        if (idx < b1) acc_elem<DT>(one, p.x, idx);
-        for (;;) {
-            if (idx < b1 && idx >= cur_start && idx < cur_end) acc.add(one);
-            if (cur_end > b0) spread = true;
-            if (cur_end >= b1) break;
-            emit_advance();
-        }
+    auto skip = [&](int64_t at) {  // skip_empty on the stream state
+        const int es = std::is_same<A, long long>::value || p.fp64 ? 8 : 4;
+        const SegWindow n = skip_empty(p.offsets, p.nseg, p.out, es, at, SegWindow{wb, win, nxt, kb});
+        wb = n.wb;
+        win = n.win;
+        nxt = n.nxt;
+        kb = n.kb;
     };
 
     // Lane l reads vector j ^ sw of its strip at step j: eight consecutive lanes
@@ -912,7 +1034,7 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
     };
 
     // the chunk of `ce` elements from c0 in ring stage `sb`, zero-filled to CHUNK bytes
-    auto chunk = [&](int ce, uint32_t sb) {
+    auto chunk = [&](const int64_t c0, int ce, uint32_t sb) {
         const uint32_t strip = sb + (uint32_t)lane * (CHUNK / 32u);
         const uint32_t v0 = strip + 16u * (uint32_t)sw;  // the strip is aligned to its size
         if (cur_end >= c0 + ce) {  // no segment ends inside the chunk
@@ -991,7 +1113,6 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
             }
             acc = RunSum<A>::of(t.total());
             spread = true;
-            cur_start = c0 + prev;
             cur_end = __shfl_sync(0xffffffffu, win, kb);
             return;
         }
@@ -1028,7 +1149,6 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
             if (!advance()) break;
             window();
         }
-        cur_start = c0 + prev;
         cur_end = __shfl_sync(0xffffffffu, win, kb);
 
         bool closes = qf < SE;
@@ -1088,71 +1208,122 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
         if (closes) seg_out(p, qseg, closed);
     };
 
+    // The walk: of each stretch the head's elements, the chunks, the tail's elements;
+    // everything before `pos` is summed.  One loop, so that the code which closes segments
+    // is there once.
     int st = 0;
     uint32_t par = 0;
-    bool bail = false;
-    const unsigned char* src = p.x + (c0 + (int64_t)S * CE) * EB;  // the next chunk to copy
-    scalar_chunk(lo, c0);
-    for (int k = 0; k < nch; ++k) {
-        if (!__all_sync(0xffffffffu, mbar_wait_bounded(bars + 8u * st, par, p.limit_ns))) {
-            if (lane == 0) {
-                atomicOr(p.err, kErrTimeout);
-                // leave no copy writing this CTA's shared memory: wait for the ones
-                // issued (chunks k .. k + S - 1), bounded separately (>= 1 s)
-                const uint64_t drain = p.limit_ns > 1000000000ull ? p.limit_ns : 1000000000ull;
-                for (int j = k; j < nch && j < k + S; ++j) {
-                    mbar_wait_bounded(bars + 8u * st, par, drain);
-                    if (++st == S) {
-                        st = 0;
-                        par ^= 1u;
-                    }
-                }
+    bool bail = false, open = true;
+    int flight = left < S ? left : S;  // copies under way when a wait expires
+    int64_t pos = lo;
+    // Many segments: long runs of empty ones may be among them, which a chunk would take a
+    // window at a time.  The piece is then walked in stretches that end where one starts.
+    bool more = far < hi && next_run(p.offsets, p.nseg, wb + kb, hi) < hi;
+    if (__builtin_expect(more, 0)) {
+        for (; flight > 0; --flight) {
+            bail = !__all_sync(0xffffffffu, mbar_wait_bounded(bars + 8u * st, par, p.limit_ns));
+            if (bail) break;
+            if (++st == S) {
+                st = 0;
+                par ^= 1u;
             }
-            bail = true;
-            break;
         }
-        const int ce = k == nch - 1 ? last_ce : CE;
-        const uint32_t sb = ring + (uint32_t)st * CHUNK;
-        if (ce < CE) {  // a short copy (the piece's last): zeros behind it
-            for (uint32_t b = (uint32_t)ce * EB + 16u * lane; b < CHUNK; b += 512u)
-                asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(sb + b), "r"(0) : "memory");
+        head = left = tail = 0;
+    }
+    while (!bail) {
+        const bool end = head + left + tail == 0;
+        while (__builtin_expect(cur_end <= pos, 0)) {  // segments that end here
+            emit_advance();
+            if (end && !more && !last) {
+                open = false;
+                break;
+            }
+            if (cur_end == pos) {
+                skip(pos);
+                cur_end = __shfl_sync(0xffffffffu, win, kb);
+            }
+        }
+        if (__builtin_expect(end, 0)) {
+            if (!more) break;
+            const int64_t to = next_run(p.offsets, p.nseg, wb + kb, stashed(4));
+            more = to < stashed(4);
+            geometry(pos, to);
+            if (lane == 0) {
+                fence_proxy_async_smem();
+                for (int j = 0; j < S; ++j)
+                    issue(p.x + (pos + head + (int64_t)j * CE) * EB, left - j, st + j < S ? st + j : st + j - S);
+            }
             __syncwarp();
+            continue;
         }
-        while (cur_end <= c0) emit_advance();
-        chunk(ce, sb);
-        __syncwarp();  // every lane has read the stage
-        if (lane == 0) {
-            fence_proxy_async_smem();
-            issue(src, k + S, st);
+        if (__builtin_expect(head > 0 || left == 0, 0)) {  // elements, at most 32, up to the open segment's end
+            int n = head > 0 ? head : tail;
+            if (cur_end - pos < n) n = (int)(cur_end - pos);
+            if (lane < n) {
+                A one = Op<A>::zero();
+                acc_elem<DT>(one, p.x, pos + lane);
+                acc.add(one);
+            }
+            spread = true;
+            if (head > 0) head -= n;
+            else tail -= n;
+            pos += n;
+            continue;
         }
-        src += CHUNK;
-        c0 += ce;
-        if (++st == S) {
-            st = 0;
-            par ^= 1u;
+        do {  // chunks, until a segment ends where one starts
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(bars + 8u * st, par, p.limit_ns))) {
+                flight = left < S ? left : S;
+                bail = true;
+                break;
+            }
+            const int ce = left == 1 ? last_ce : CE;
+            const uint32_t sb = ring + (uint32_t)st * CHUNK;
+            if (ce < CE) {  // a short copy (the piece's last): zeros behind it
+                for (uint32_t b = (uint32_t)ce * EB + 16u * lane; b < CHUNK; b += 512u)
+                    asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(sb + b), "r"(0) : "memory");
+                __syncwarp();
+            }
+            chunk(pos, ce, sb);
+            __syncwarp();  // every lane has read the stage
+            if (lane == 0) {
+                fence_proxy_async_smem();
+                issue(p.x + (pos + (int64_t)S * CE) * EB, left - S, st);
+            }
+            pos += ce;
+            --left;
+            if (++st == S) {
+                st = 0;
+                par ^= 1u;
+            }
+        } while (left > 0 && cur_end > pos);
+    }
+    if (bail && lane == 0) {
+        atomicOr(p.err, kErrTimeout);
+        // leave no copy writing this CTA's shared memory: wait for the ones under way,
+        // bounded separately (>= 1 s)
+        const uint64_t drain = p.limit_ns > 1000000000ull ? p.limit_ns : 1000000000ull;
+        for (; flight > 0; --flight) {
+            mbar_wait_bounded(bars + 8u * st, par, drain);
+            if (++st == S) {
+                st = 0;
+                par ^= 1u;
+            }
         }
     }
     int64_t spanning = -1;  // the owned segment that runs past this piece
     if (!bail) {            // a timeout's results are void (SR_ERR_TIMEOUT): nothing left to finish
-        scalar_chunk(c0, hi);
-        const int64_t next_lo = (w == Wn - 1) ? INT64_MAX : base + (w + 1) * E;
-        // the segment holding the piece's last element, then any (empty) segment
-        // this warp owns that starts at or after hi
-        while (wb + kb <= p.nseg && cur_start < next_lo) {
-            if (cur_end <= hi || cont) {
-                emit_advance();
-                continue;
-            }
-            spanning = wb + kb - 1;  // owned, runs past this piece
+        if (cont) {  // the whole piece lies inside an earlier warp's segment
+            emit_first(wb + kb - 1, take_acc());
+        } else if (open && wb + kb <= p.nseg) {
+            spanning = wb + kb - 1;
             const A v = take_acc();
             if (p.stage == kStageAtomic) {
                 if (lane == 0) seg_atomic(p, spanning, v);
             } else {
                 if (lane == 0) carry_store(p, p.carry_last, w, v);
                 if (p.stage == kStageLastBlock)
-                    span_arrive<A, true>(p, spanning, w, (cur_end - 1 - base) / E, lane);
+                    span_arrive<A, true>(p, spanning, w, (cur_end - 1 - stashed(0)) / stashed(2), lane);
             }
-            break;  // the next segment starts in the next warp's piece
         }
     }
 
@@ -1168,7 +1339,7 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
         g.sync();
         if (spanning >= 0) {
             const int64_t end = __ldg(p.offsets + spanning + 1);
-            finish_span<A, true>(p, spanning, w, (end - 1 - base) / E, lane);
+            finish_span<A, true>(p, spanning, w, (end - 1 - stashed(0)) / stashed(2), lane);
         }
     }
 }
