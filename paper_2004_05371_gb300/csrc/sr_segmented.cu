@@ -183,7 +183,9 @@ int seg_plan(int64_t nseg, int dtype, const sr_config& c, const DeviceInfo& d, S
             (c.block_threads && c.block_threads != 256))
             return SR_ERR_UNSUPPORTED;
         if (c.grid > (int64_t)kAdaptMaxCtasPerSm * d.sms) return SR_ERR_LAUNCH;
-        p.stage = SR_LAST_BLOCK;  // the stage bits are ignored
+        // The stage bits are ignored: tickets, but for int32 without the flag, which keeps
+        // the atomic finish from above (4096 segments of 256 in us: 10.7 with tickets, 8.2).
+        if (dtype != SR_I32 || (c.variant & SR_F_ADAPTIVE_SEGMENTS)) p.stage = SR_LAST_BLOCK;
         p.block = 256;
         p.cta = kTmaBlock;
         p.stages = 2;
