@@ -307,8 +307,8 @@ int seg_launch(const void* x, const int64_t* offsets, void* out, const SegPlan& 
     if (p.stage == SR_TWO_KERNEL && !p.warp && !p.lane) {
         int64_t wn = p.warps;
         int pv = p.vec / elem_size(p.dtype);
-        int e_min = p.bulk ? p.unroll * 32 * pv / kPieceParts : pv;  // the first kernel's smallest piece
-        void* fargs[] = {&kp, &wn, &pv, &e_min};
+        int chunk = p.bulk ? p.unroll * 32 * pv : 0;  // elements of the TMA form's chunks
+        void* fargs[] = {&kp, &wn, &pv, &chunk};
         lc.gridDim = dim3((unsigned)((p.warps * 32 + 255) / 256));
         lc.blockDim = dim3(256);
         e = cudaLaunchKernelExC(&lc, p.fin, fargs);

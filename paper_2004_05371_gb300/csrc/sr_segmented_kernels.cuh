@@ -230,9 +230,10 @@ template <> struct RunSum<float> {
 // registers (10,000 lognormal segments at 32 B x 4: 168 -> 205 us).
 template <class P, bool WIDE> __device__ __forceinline__ void finish_span_typed(const SegParams& p, int64_t s,
                                                                                 int64_t w_o, int64_t w_e, int lane) {
-    P acc = Op<P>::zero();
+    P acc = Op<P>::zero(), own = Op<P>::zero();
     int64_t w = w_o + 1 + lane;
     if constexpr (WIDE) {
+        own = carry_load<P>(p.carry_last, w_o);  // one trip together with the others
         RunSum<P> sum = RunSum<P>::of(acc);
         for (; w + 7 * 32 <= w_e; w += 8 * 32) {
             P c[8];
@@ -247,7 +248,7 @@ template <class P, bool WIDE> __device__ __forceinline__ void finish_span_typed(
     }
     acc = warp_reduce(acc);
     if (lane == 0) {
-        P total = Op<P>::add(carry_load<P>(p.carry_last, w_o), acc);
+        P total = Op<P>::add(WIDE ? own : carry_load<P>(p.carry_last, w_o), acc);
         if constexpr (std::is_same<P, double>::value) seg_out_d(p, s, total);
         else seg_out(p, s, total);
     }
@@ -709,6 +710,11 @@ template <int EB> __device__ __forceinline__ void keep_from(uint32_t (&r)[4], in
     }
 }
 
+// Smallest piece of a warp, in elements of `eb` bytes, for chunks of `ce` (sr_segparams.h).
+__device__ __forceinline__ int64_t strip_min_piece(int64_t n, int64_t nseg, int ce, int eb) {
+    return n * eb >= (int64_t)kLongMean * nseg ? ce : ce / kPieceParts;
+}
+
 // Offsets fetched into L2 this far ahead of the window: the one after `nxt`.  Further
 // ahead they are more often gone again (16M x 16 f32: 211 us with 64, 216 with 192,
 // 231 with 256).
@@ -838,7 +844,8 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
     const int64_t N = __ldg(p.offsets + p.nseg) - base;
     int64_t E = (N + Wn - 1) / Wn;
     E = ((E + PV - 1) / PV) * PV;
-    if (E < CE / kPieceParts) E = CE / kPieceParts;
+    const int64_t e_min = strip_min_piece(N, p.nseg, CE, EB);
+    if (E < e_min) E = e_min;
     const int64_t lo = base + (w * E < N ? w * E : N);
     const int64_t hi = base + ((w + 1) * E < N ? (w + 1) * E : N);
 
@@ -905,8 +912,13 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
     // offsets[wb + k] in win and offsets[wb + 32 + k] in nxt (loaded one window
     // ahead).  Entry kb is the end of the open segment, wb + kb - 1.
     const int64_t at = N > 0 ? (int64_t)((float)(w * E) / (float)N * (float)p.nseg) : 0;
-    const int r0 =
-        (int)(warp_search(p.offsets, p.nseg, base + w * E, at < p.nseg ? at : p.nseg, lane, wb, win, fill) - wb);
+    int r0 = 0;
+    if (w * E <= N) {
+        r0 = (int)(warp_search(p.offsets, p.nseg, base + w * E, at < p.nseg ? at : p.nseg, lane, wb, win, fill) - wb);
+    } else {  // nothing for this warp: past the last segment
+        wb = p.nseg;
+        win = far = INT64_MAX;
+    }
     int64_t nxt = (wb + 32 + lane <= p.nseg) ? __ldg(p.offsets + wb + 32 + lane) : INT64_MAX;
     // the open segment began in an earlier warp's piece
     bool cont = lo < hi && __shfl_sync(0xffffffffu, win, r0) > lo;
@@ -1346,7 +1358,7 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
 
 // Second kernel of the two-kernel form: one warp per first-kernel warp.
 template <int DT, bool COMP>
-__global__ void __launch_bounds__(256) seg_finish_kernel(const SegParams p, int64_t Wn, int PV, int e_min) {
+__global__ void __launch_bounds__(256) seg_finish_kernel(const SegParams p, int64_t Wn, int PV, int chunk) {
     using A = typename Acc<DT, COMP>::T;
     grid_dependency_wait();  // the implicit barrier: every first-kernel warp has finished
     allow_dependents();
@@ -1360,6 +1372,7 @@ __global__ void __launch_bounds__(256) seg_finish_kernel(const SegParams p, int6
     const int64_t N = __ldg(p.offsets + p.nseg) - base;
     int64_t E = (N + Wn - 1) / Wn;  // the first kernel's piece size
     E = ((E + PV - 1) / PV) * PV;
+    const int64_t e_min = chunk ? strip_min_piece(N, p.nseg, chunk, SegElem<DT>::v) : PV;
     if (E < e_min) E = e_min;
     const int64_t end = __ldg(p.offsets + s + 1);
     finish_span<A, true>(p, s, w, (end - 1 - base) / E, lane);

@@ -15,8 +15,13 @@ constexpr int kErrBadOffsets = 4;  // the checked entry found offsets it may not
 constexpr int kStripTableBytes = 128;
 // TMA form: a warp's piece is at least a chunk / kPieceParts, so the segments of
 // a small input seldom cross a warp (100 segments of 30 elements: 8.3 us with
-// pieces down to one vector, 6.9 now).
+// pieces down to one vector, 6.9 now), and a whole chunk where segments average
+// kLongMean bytes or more: a chunk then costs the same instructions however much of
+// it is there, and more warps only add to them (4096 segments of 256 f32: 10.4 us
+// with quarters, 9.0; equal ones 10.7, 5.3).  Shorter ones are summed by single
+// lanes, for which whole chunks are too few warps (40,000 of 2: 5.2 us, 10.1).
 constexpr int kPieceParts = 4;
+constexpr int kLongMean = 128;
 
 // Kernel argument block of the segmented sum (sr_segmented_kernels.cuh).
 struct SegParams {
