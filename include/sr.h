@@ -223,8 +223,11 @@ int sr_reduce_sum(const void* x, int64_t n, int dtype, void* out, int variant,
 
 /* End-to-end form: x and out are HOST pointers (x preferably page-locked, e.g.
  * cudaHostAlloc / cudaHostRegister, so copies run asynchronously).  With stage
- * SR_AUTO a page-locked array of at most 128 MiB is read in place, as with
- * SR_F_HOST_DIRECT; otherwise the input is copied to the device in 64 MiB chunks through two library-owned staging
+ * SR_AUTO a page-locked array of at most 128 MiB that lies in one allocation
+ * or registration is read in place, as with SR_F_HOST_DIRECT (the kernel then
+ * holds the SMs for the link's time, up to 0.65 ms, and a sum may round
+ * differently from that of the same data in pageable memory); otherwise the
+ * input is copied to the device in 64 MiB chunks through two library-owned staging
  * buffers on two copy streams, each chunk reduced on `stream` while the next
  * one is copied (the chunk units' partials go to disjoint workspace slots),
  * and one final kernel combines all partials in order.  The result comes back

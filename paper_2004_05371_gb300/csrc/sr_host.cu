@@ -7,8 +7,8 @@
 // form), and one final kernel reduces all slots in order.  Copy of chunk k+1
 // overlaps the reduction of chunk k.
 //
-// A page-locked array of at most two chunks is read in place by one kernel
-// instead: with so little to overlap, the copy, its events and the launches after it
+// A page-locked array of at most two chunks, within one allocation or registration, is
+// read in place by one kernel instead: with so little to overlap, the copy, its events and the launches after it
 // cost more than they hide (link 210 GB/s either way; pipeline / in place, us:
 // 4 KiB 23 / 16, 1 MiB 31 / 21, 16 MiB 112 / 97, 64 MiB 353 / 335, 128 MiB 676 / 653).  Above, the
 // pipeline stays within 2 % and leaves the SMs to other streams.
@@ -22,6 +22,9 @@
 #include <mutex>
 #include <utility>
 
+#include <cuda.h>  // types of the driver's pointer query (fetched at run time)
+
+#include "sr_hostrange.h"
 #include "sr_internal.h"
 
 namespace sr {
@@ -120,15 +123,35 @@ int result_slot(HostPipe* hp, unsigned char** host, void** dev) {
     return e == cudaSuccess ? SR_OK : status_from_cuda(e);
 }
 
-// Whether [x, x + bytes) starts and ends in page-locked memory that the device can read.
-bool page_locked(const void* x, size_t bytes) {
-    cudaPointerAttributes a, b;
-    if (cudaPointerGetAttributes(&a, x) != cudaSuccess ||
-        cudaPointerGetAttributes(&b, static_cast<const unsigned char*>(x) + bytes - 1) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return a.type == cudaMemoryTypeHost && b.type == cudaMemoryTypeHost && a.devicePointer && b.devicePointer;
+// The driver's view of one host address (no page-locked memory where it has none to give).
+HostRange query_host(uintptr_t at) {
+    using Fn = CUresult (*)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+    static const Fn get = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+            r != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<Fn>(f);
+    }();
+    HostRange h;
+    if (!get) return h;
+    CUmemorytype type = (CUmemorytype)0;
+    CUdeviceptr device = 0, start = 0;
+    size_t size = 0;
+    int managed = 0;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                  CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE,
+                                  CU_POINTER_ATTRIBUTE_IS_MANAGED};
+    void* data[] = {&type, &device, &start, &size, &managed};
+    if (get(5, what, data, (CUdeviceptr)at) != CUDA_SUCCESS) return h;
+    h.page_locked = type == CU_MEMORYTYPE_HOST && !managed && device;
+    h.start = (uintptr_t)start;
+    h.size = size;
+    h.device = (uintptr_t)device;
+    return h;
 }
 
 // The reduction reads the host array in place (no staging copies).
@@ -207,7 +230,8 @@ extern "C" int sr_reduce_sum_host(const void* host_x, int64_t n, int dtype, void
     if (st != SR_OK) return st;
     const int es = elem_size(dtype);
     const size_t bytes = (size_t)n * es;
-    if (stage == SR_AUTO && bytes > 0 && bytes <= kInPlaceBytes && page_locked(host_x, bytes)) {
+    if (stage == SR_AUTO && bytes > 0 && bytes <= kInPlaceBytes &&
+        one_page_locked_range(reinterpret_cast<uintptr_t>(host_x), bytes, query_host)) {
         c.variant &= ~SR_STAGE_MASK;
         return host_direct(host_x, n, dtype, host_out, c, stream);
     }
