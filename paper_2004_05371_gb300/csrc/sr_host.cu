@@ -123,34 +123,46 @@ int result_slot(HostPipe* hp, unsigned char** host, void** dev) {
     return e == cudaSuccess ? SR_OK : status_from_cuda(e);
 }
 
+// A driver function by name (nullptr where there is none).
+template <class Fn> Fn driver_function(const char* name) {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult r;
+    if (cudaGetDriverEntryPointByVersion(name, &f, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+        r != cudaDriverEntryPointSuccess) {
+        cudaGetLastError();
+        f = nullptr;
+    }
+    return reinterpret_cast<Fn>(f);
+}
+
 // The driver's view of one host address (no page-locked memory where it has none to give).
 HostRange query_host(uintptr_t at) {
-    using Fn = CUresult (*)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
-    static const Fn get = [] {
-        void* f = nullptr;
-        cudaDriverEntryPointQueryResult r;
-        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &r) != cudaSuccess ||
-            r != cudaDriverEntryPointSuccess) {
-            cudaGetLastError();
-            f = nullptr;
-        }
-        return reinterpret_cast<Fn>(f);
-    }();
+    static const auto get =
+        driver_function<CUresult (*)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr)>("cuPointerGetAttributes");
+    static const auto current = driver_function<CUresult (*)(CUcontext*)>("cuCtxGetCurrent");
     HostRange h;
-    if (!get) return h;
-    CUmemorytype type = (CUmemorytype)0;
-    CUdeviceptr device = 0, start = 0;
+    if (!get || !current) return h;
+    // The driver answers only with a context current: a thread's first calls of the runtime
+    // need not have made one so (with one, it stays the caller's).
+    CUcontext ctx = nullptr;
+    int dev = 0;
+    if (current(&ctx) != CUDA_SUCCESS) return h;
+    cudaPointerAttributes a;
+    if ((!ctx && (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess)) ||
+        cudaPointerGetAttributes(&a, reinterpret_cast<const void*>(at)) != cudaSuccess) {
+        cudaGetLastError();
+        return h;
+    }
+    if (a.type != cudaMemoryTypeHost || !a.devicePointer) return h;
+    CUdeviceptr start = 0;
     size_t size = 0;
-    int managed = 0;
-    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
-                                  CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE,
-                                  CU_POINTER_ATTRIBUTE_IS_MANAGED};
-    void* data[] = {&type, &device, &start, &size, &managed};
-    if (get(5, what, data, (CUdeviceptr)at) != CUDA_SUCCESS) return h;
-    h.page_locked = type == CU_MEMORYTYPE_HOST && !managed && device;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* data[] = {&start, &size};
+    if (get(2, what, data, (CUdeviceptr)at) != CUDA_SUCCESS) return h;
+    h.page_locked = true;
     h.start = (uintptr_t)start;
     h.size = size;
-    h.device = (uintptr_t)device;
+    h.device = reinterpret_cast<uintptr_t>(a.devicePointer);
     return h;
 }
 
