@@ -16,7 +16,7 @@
 // The result is written by the kernel into page-locked memory of the library's
 // (a copy back to the device's caller took another 8 us).
 #include <algorithm>
-#include <atomic>
+#include <condition_variable>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -32,7 +32,7 @@ namespace {
 
 constexpr size_t kChunkBytes = 64u << 20;
 constexpr size_t kInPlaceBytes = 2 * kChunkBytes;  // page-locked arrays up to here are read in place
-constexpr unsigned kResultSlots = 64;              // 64 bytes apart; calls take them in turn
+constexpr int kResultSlots = 64;  // 64 bytes apart; a call holds one until its value is copied out
 
 struct HostPipe {
     unsigned char* stage[2] = {nullptr, nullptr};
@@ -41,7 +41,8 @@ struct HostPipe {
     cudaEvent_t consumed[2] = {nullptr, nullptr};
     size_t chunk = 0;
     unsigned char* result = nullptr;  // kResultSlots page-locked slots, host and device address alike
-    std::atomic<unsigned> next{0};
+    uint64_t busy = 0;                // slots held (under g_hp_mu)
+    std::condition_variable freed;
 };
 
 std::mutex g_hp_mu;
@@ -116,12 +117,40 @@ using namespace sr;
 
 namespace {
 
-// The device address of the next result slot (the host's too, in *host).
-int result_slot(HostPipe* hp, unsigned char** host, void** dev) {
-    *host = hp->result + 64 * (size_t)(hp->next.fetch_add(1, std::memory_order_relaxed) % kResultSlots);
-    const cudaError_t e = cudaHostGetDevicePointer(dev, *host, 0);
-    return e == cudaSuccess ? SR_OK : status_from_cuda(e);
-}
+// A result slot of the pipe, this call's alone until it returns: with more calls than slots
+// blocked on one stream, the others wait for one (before, they took the slots in turn, and
+// an earlier call could find a later one's sum in its own).
+class ResultSlot {
+public:
+    explicit ResultSlot(HostPipe* hp) : hp_(hp) {
+        std::unique_lock<std::mutex> lk(g_hp_mu);
+        hp_->freed.wait(lk, [&] { return ~hp_->busy != 0; });
+        for (k_ = 0; (hp_->busy >> k_) & 1; ++k_) {
+        }
+        hp_->busy |= uint64_t(1) << k_;
+        host = hp_->result + 64 * (size_t)k_;
+        const cudaError_t e = cudaHostGetDevicePointer(&dev, host, 0);
+        status = e == cudaSuccess ? SR_OK : status_from_cuda(e);
+    }
+    ~ResultSlot() {
+        {
+            std::lock_guard<std::mutex> lk(g_hp_mu);
+            hp_->busy &= ~(uint64_t(1) << k_);
+        }
+        hp_->freed.notify_one();
+    }
+    ResultSlot(const ResultSlot&) = delete;
+    ResultSlot& operator=(const ResultSlot&) = delete;
+
+    unsigned char* host = nullptr;
+    void* dev = nullptr;
+    int status = SR_OK;
+
+private:
+    HostPipe* hp_;
+    int k_ = 0;
+};
+static_assert(kResultSlots == 64, "one bit per slot");
 
 // A driver function by name (nullptr where there is none).
 template <class Fn> Fn driver_function(const char* name) {
@@ -205,15 +234,13 @@ int host_direct(const void* host_x, int64_t n, int dtype, void* host_out, sr_con
     HostPipe* hp = nullptr;
     st = get_pipe(s, 0, &hp);
     if (st != SR_OK) return st;
-    unsigned char* slot = nullptr;
-    void* dev_out = nullptr;
-    st = result_slot(hp, &slot, &dev_out);
-    if (st != SR_OK) return st;
-    st = reduce_launch(dx, dev_out, p, *d, ws, s);
+    ResultSlot slot(hp);
+    if (slot.status != SR_OK) return slot.status;
+    st = reduce_launch(dx, slot.dev, p, *d, ws, s);
     if (st != SR_OK) return st;
     cudaError_t e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return status_from_cuda(e);
-    std::memcpy(host_out, slot, (dtype == SR_I32 || p.fp64) ? 8 : 4);
+    std::memcpy(host_out, slot.host, (dtype == SR_I32 || p.fp64) ? 8 : 4);
     return SR_OK;
 }
 
@@ -259,10 +286,8 @@ extern "C" int sr_reduce_sum_host(const void* host_x, int64_t n, int dtype, void
     if (st != SR_OK) return st;
 
     const bool fp64 = (c.variant & SR_F_FP64_COMBINE) && dtype != SR_I32;
-    unsigned char* result = nullptr;
-    void* dev_out = nullptr;
-    st = result_slot(hp, &result, &dev_out);
-    if (st != SR_OK) return st;
+    ResultSlot result(hp);
+    if (result.status != SR_OK) return result.status;
     int slot = 0;
     Plan last;
     bool have_plan = false;
@@ -290,7 +315,7 @@ extern "C" int sr_reduce_sum_host(const void* host_x, int64_t n, int dtype, void
         if (slot + p.units > kMaxUnits) return SR_ERR_ARG;
         Workspace wk = ws;
         wk.partials = ws.partials + (size_t)slot * kSlotBytes;
-        st = reduce_launch(hp->stage[b], dev_out, p, *d, wk, s, /*skip_final=*/true);
+        st = reduce_launch(hp->stage[b], result.dev, p, *d, wk, s, /*skip_final=*/true);
         if (st != SR_OK) return st;
         slot += p.units;
         last = p;
@@ -301,10 +326,10 @@ extern "C" int sr_reduce_sum_host(const void* host_x, int64_t n, int dtype, void
         if (len == 0) break;
     }
     if (!have_plan) return SR_ERR_ARG;
-    st = reduce_launch_final(last, slot, dev_out, ws, s);
+    st = reduce_launch_final(last, slot, result.dev, ws, s);
     if (st != SR_OK) return st;
     const cudaError_t e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return status_from_cuda(e);
-    std::memcpy(host_out, result, (dtype == SR_I32 || fp64) ? 8 : 4);
+    std::memcpy(host_out, result.host, (dtype == SR_I32 || fp64) ? 8 : 4);
     return SR_OK;
 }
