@@ -43,6 +43,7 @@ struct HostPipe {
     unsigned char* result = nullptr;  // kResultSlots page-locked slots, host and device address alike
     uint64_t busy = 0;                // slots held (under g_hp_mu)
     std::condition_variable freed;
+    std::mutex copying;               // held by the call that uses the staging buffers and events
 };
 
 std::mutex g_hp_mu;
@@ -281,7 +282,12 @@ extern "C" int sr_reduce_sum_host(const void* host_x, int64_t n, int dtype, void
         chunk = (bytes + max_chunks - 1) / max_chunks;
         chunk = (chunk + (1u << 20) - 1) & ~((size_t)(1u << 20) - 1);
     }
+    // One call at a time copies through a stream's staging buffers: with two, the second
+    // one's copies, which its own stream orders behind nothing, overwrote the first one's.
     HostPipe* hp = nullptr;
+    st = get_pipe(s, 0, &hp);
+    if (st != SR_OK) return st;
+    std::lock_guard<std::mutex> copying(hp->copying);
     st = get_pipe(s, chunk, &hp);
     if (st != SR_OK) return st;
 

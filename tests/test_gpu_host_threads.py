@@ -9,7 +9,7 @@ import torch
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("variant_name", ["AUTO", "F_HOST_DIRECT"])
+@pytest.mark.parametrize("variant_name", ["AUTO", "F_HOST_DIRECT", "TWO_KERNEL"])  # the last by copies
 def test_two_hundred_threads_on_one_stream(sr, variant_name):
     threads, n = 200, 1 << 12
     stream = torch.cuda.Stream()
