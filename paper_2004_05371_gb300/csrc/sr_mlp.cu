@@ -549,17 +549,20 @@ int sr_mlp_train_step(sr_mlp h, const float* X, const float* Q, int batch, float
     const int parts = (int)std::min<int64_t>(((int64_t)batch + kTile - 1) / kTile, 2 * di->sms);
     cudaError_t e;
     if (parts > h->max_parts) {
+        // room for every batch up to the next multiple of 16, so that a step captured
+        // after one of a slightly smaller batch need not allocate
+        const int room = (int)std::min<int64_t>(2 * (((int64_t)batch + 15) / 16), 2 * di->sms);
         cudaFree(h->partial);
         cudaFree(h->loss_partial);
         h->partial = nullptr;
         h->loss_partial = nullptr;
-        e = cudaMalloc(&h->partial, sizeof(float) * (size_t)parts * h->d.P);
-        if (e == cudaSuccess) e = cudaMalloc(&h->loss_partial, sizeof(float) * parts);
+        e = cudaMalloc(&h->partial, sizeof(float) * (size_t)room * h->d.P);
+        if (e == cudaSuccess) e = cudaMalloc(&h->loss_partial, sizeof(float) * room);
         if (e != cudaSuccess) {
             h->max_parts = 0;
             return status_from_cuda(e);
         }
-        h->max_parts = parts;
+        h->max_parts = room;
     }
     const size_t smem = sizeof(float) * (size_t)grad_smem(h->d).total;
     st = prepare_function((const void*)mlp_grad_kernel, smem, false);
