@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(kGradThreads, 2) mlp_grad_kernel(MlpDims d, co
     float gb[3] = {};                                   // thread t < 64: entry t of b1, b2, b3
     float loss = 0.f;                                   // thread 0
     const float invB = 1.0f / (float)B;
-    const int tiles = (B + kTile - 1) / kTile;
+    const int tiles = (B - 1) / kTile + 1;  // B + kTile - 1 may not fit
     __syncthreads();
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         const int b0 = tile * kTile, nb = min(kTile, B - b0);
