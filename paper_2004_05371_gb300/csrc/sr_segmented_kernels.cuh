@@ -864,10 +864,10 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
     };
     geometry(lo, hi);
     // segments that start at hi are this warp's too (elsewhere they are the next one's)
-    const bool last = w == Wn - 1 || base + (w + 1) * E > hi;
-    // base, E and hi are wanted only where a segment crosses the piece's ends or a stretch
-    // ends: the lanes keep a word each of them
-    const uint32_t stash = (uint32_t)((lane & 4 ? hi : lane & 2 ? E : base) >> (lane & 1 ? 32 : 0));
+    const int64_t last = w == Wn - 1 || base + (w + 1) * E > hi;
+    // base, E, hi and last are wanted only where a segment crosses the piece's ends or a
+    // stretch ends: the lanes keep a word each of them
+    const uint32_t stash = (uint32_t)((lane & 4 ? (lane & 2 ? last : hi) : lane & 2 ? E : base) >> (lane & 1 ? 32 : 0));
     auto stashed = [&](int at) {
         return (int64_t)((uint64_t)__shfl_sync(0xffffffffu, stash, at) |
                          (uint64_t)__shfl_sync(0xffffffffu, stash, at + 1) << 32);
@@ -1225,7 +1225,7 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
     // is there once.
     int st = 0;
     uint32_t par = 0;
-    bool bail = false, open = true;
+    bool bail = false;
     int flight = left < S ? left : S;  // copies under way when a wait expires
     int64_t pos = lo;
     // Many segments: long runs of empty ones may be among them, which a chunk would take a
@@ -1246,8 +1246,9 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
         const bool end = head + left + tail == 0;
         while (__builtin_expect(cur_end <= pos, 0)) {  // segments that end here
             emit_advance();
-            if (end && !more && !last) {
-                open = false;
+            if (end && !more && !stashed(6)) {
+                wb = p.nseg;  // nothing open: past the last segment
+                kb = 1;
                 break;
             }
             if (cur_end == pos) {
@@ -1326,7 +1327,7 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
     if (!bail) {            // a timeout's results are void (SR_ERR_TIMEOUT): nothing left to finish
         if (cont) {  // the whole piece lies inside an earlier warp's segment
             emit_first(wb + kb - 1, take_acc());
-        } else if (open && wb + kb <= p.nseg) {
+        } else if (wb + kb <= p.nseg) {
             spanning = wb + kb - 1;
             const A v = take_acc();
             if (p.stage == kStageAtomic) {
