@@ -19,9 +19,11 @@ constexpr int kStripTableBytes = 128;
 // kLongMean bytes or more: a chunk then costs the same instructions however much of
 // it is there, and more warps only add to them (4096 segments of 256 f32: 10.4 us
 // with quarters, 9.0; equal ones 10.7, 5.3).  Shorter ones are summed by single
-// lanes, for which whole chunks are too few warps (40,000 of 2: 5.2 us, 10.1).
+// lanes, for which whole chunks are too few warps (40,000 of 2: 5.2 us, 10.1; at a
+// mean of 136 bytes 4096 to 7000 segments lose 3-9 % and 12,000 gain 2-14 %, at 168
+// all but 4096 int32 ones gain).
 constexpr int kPieceParts = 4;
-constexpr int kLongMean = 128;
+constexpr int kLongMean = 160;
 
 // Kernel argument block of the segmented sum (sr_segmented_kernels.cuh).
 struct SegParams {

@@ -1,5 +1,5 @@
 """Small segmented calls: the strip kernel's smallest piece (a whole chunk from a
-mean of 128 bytes per segment, a quarter below) either side of the line, in
+mean of 160 bytes per segment, a quarter below) either side of the line, in
 every finish, results exact; and the default form's time against the LDG
 kernel's on the same call, where the pieces decide it."""
 import numpy as np
@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("dtype,eb", [(torch.int32, 4), (torch.float32, 4), (torch.bfloat16, 2), (torch.uint8, 1)])
 def test_either_side_of_the_mean(sr, dtype, eb):
     for nseg in (1, 7, 300, 5000):
-        for total in (128 * nseg // eb - 1, 128 * nseg // eb, 128 * nseg // eb + 1, 40 * nseg):
+        for total in (160 * nseg // eb - 1, 160 * nseg // eb, 160 * nseg // eb + 1, 30 * nseg):
             rng = np.random.default_rng(total)
             cuts = np.sort(rng.integers(0, total + 1, nseg - 1))
             off = np.concatenate([[0], cuts, [total]]).astype(np.int64)
