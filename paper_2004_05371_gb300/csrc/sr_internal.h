@@ -97,7 +97,7 @@ inline int elem_size(int dtype) { return dtype == SR_BF16 ? 2 : (dtype == SR_FP8
 // small kernel launched with programmatic stream serialisation, ordered after
 // the stream's previous work (sr_reduce.cu).  Used where the atomic finish
 // needs a zeroed output: a memset node costs several microseconds more.
-int launch_zero(void* p, size_t bytes, cudaStream_t s);
+int launch_zero(void* p, size_t bytes, cudaStream_t s, bool late = false);
 
 // Configuration and persisted selection state (sr_persist.cu)
 // The identity a device's persisted entries are keyed by: "<SMs> <driver

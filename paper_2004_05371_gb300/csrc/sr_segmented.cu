@@ -277,9 +277,11 @@ int seg_launch(const void* x, const int64_t* offsets, void* out, const SegPlan& 
     kp.stage = p.stage;
     kp.fp64 = p.fp64 ? 1 : 0;
     cudaError_t e;
+    // the small kernel before or after lets a strip kernel of three CTAs per SM in late
+    const bool late = p.bulk && p.cta <= 256;
     if (p.stage == SR_ATOMIC && !p.warp && !p.lane) {
         const size_t ob = (p.dtype == SR_I32 || p.fp64) ? 8 : 4;
-        const int zs = launch_zero(out, ob * (size_t)p.nseg, s);
+        const int zs = launch_zero(out, ob * (size_t)p.nseg, s, late);
         if (zs != SR_OK) return zs;
     }
     void* args[] = {&kp};
@@ -308,7 +310,8 @@ int seg_launch(const void* x, const int64_t* offsets, void* out, const SegPlan& 
         int64_t wn = p.warps;
         int pv = p.vec / elem_size(p.dtype);
         int chunk = p.bulk ? p.unroll * 32 * pv : 0;  // elements of the TMA form's chunks
-        void* fargs[] = {&kp, &wn, &pv, &chunk};
+        int late_arg = late;
+        void* fargs[] = {&kp, &wn, &pv, &chunk, &late_arg};
         lc.gridDim = dim3((unsigned)((p.warps * 32 + 255) / 256));
         lc.blockDim = dim3(256);
         e = cudaLaunchKernelExC(&lc, p.fin, fargs);

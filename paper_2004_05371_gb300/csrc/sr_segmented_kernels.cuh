@@ -710,9 +710,12 @@ template <int EB> __device__ __forceinline__ void keep_from(uint32_t (&r)[4], in
     }
 }
 
-// Smallest piece of a warp, in elements of `eb` bytes, for chunks of `ce` (sr_segparams.h).
-__device__ __forceinline__ int64_t strip_min_piece(int64_t n, int64_t nseg, int ce, int eb) {
-    return n * eb >= (int64_t)kLongMean * nseg ? ce : ce / kPieceParts;
+// A warp's piece, e elements of `eb` bytes in an even split, as large as it has to be for
+// chunks of `ce` (sr_segparams.h).  From three quarters of a chunk on the even split stays:
+// fewer warps then save nothing (4096 segments of 775 f32: 10.2 us, 10.0).
+__device__ __forceinline__ int64_t strip_piece(int64_t e, int64_t n, int64_t nseg, int ce, int eb) {
+    if (n * eb >= (int64_t)kLongMean * nseg) return e < ce / 4 * 3 ? ce : e;
+    return e < ce / kPieceParts ? ce / kPieceParts : e;
 }
 
 // Offsets fetched into L2 this far ahead of the window: the one after `nxt`.  Further
@@ -844,8 +847,7 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
     const int64_t N = __ldg(p.offsets + p.nseg) - base;
     int64_t E = (N + Wn - 1) / Wn;
     E = ((E + PV - 1) / PV) * PV;
-    const int64_t e_min = strip_min_piece(N, p.nseg, CE, EB);
-    if (E < e_min) E = e_min;
+    E = strip_piece(E, N, p.nseg, CE, EB);
     const int64_t lo = base + (w * E < N ? w * E : N);
     const int64_t hi = base + ((w + 1) * E < N ? (w + 1) * E : N);
 
@@ -1359,10 +1361,14 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
 
 // Second kernel of the two-kernel form: one warp per first-kernel warp.
 template <int DT, bool COMP>
-__global__ void __launch_bounds__(256) seg_finish_kernel(const SegParams p, int64_t Wn, int PV, int chunk) {
+__global__ void __launch_bounds__(256) seg_finish_kernel(const SegParams p, int64_t Wn, int PV, int chunk,
+                                                          int late) {
     using A = typename Acc<DT, COMP>::T;
     grid_dependency_wait();  // the implicit barrier: every first-kernel warp has finished
-    allow_dependents();
+    // The next call's first kernel is let in at once, but (late) at the end where its CTAs
+    // are three to an SM: while these here hold an SM they come in unevenly (4M lognormal
+    // segments, strip kernel of 256 threads: 221 us a call, 189; two to an SM: no change).
+    if (!late) allow_dependents();
     if (p.bad != nullptr && __ldcg(p.bad) != 0) return;
     const int lane = threadIdx.x & 31;
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1373,8 +1379,8 @@ __global__ void __launch_bounds__(256) seg_finish_kernel(const SegParams p, int6
     const int64_t N = __ldg(p.offsets + p.nseg) - base;
     int64_t E = (N + Wn - 1) / Wn;  // the first kernel's piece size
     E = ((E + PV - 1) / PV) * PV;
-    const int64_t e_min = chunk ? strip_min_piece(N, p.nseg, chunk, SegElem<DT>::v) : PV;
-    if (E < e_min) E = e_min;
+    if (E < PV) E = PV;
+    if (chunk) E = strip_piece(E, N, p.nseg, chunk, SegElem<DT>::v);
     const int64_t end = __ldg(p.offsets + s + 1);
     finish_span<A, true>(p, s, w, (end - 1 - base) / E, lane);
 }

@@ -15,7 +15,8 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("dtype,eb", [(torch.int32, 4), (torch.float32, 4), (torch.bfloat16, 2), (torch.uint8, 1)])
 def test_either_side_of_the_mean(sr, dtype, eb):
     for nseg in (1, 7, 300, 5000):
-        for total in (160 * nseg // eb - 1, 160 * nseg // eb, 160 * nseg // eb + 1, 30 * nseg):
+        for total in (160 * nseg // eb - 1, 160 * nseg // eb, 160 * nseg // eb + 1, 30 * nseg,
+                      3648 * 3072 // eb - 5, 3648 * 3072 // eb + 3000):  # three quarters of a chunk to a warp
             rng = np.random.default_rng(total)
             cuts = np.sort(rng.integers(0, total + 1, nseg - 1))
             off = np.concatenate([[0], cuts, [total]]).astype(np.int64)
