@@ -932,7 +932,7 @@ __global__ void __maxnreg__(80) seg_strip_kernel(const SegParams p) {
     RunSum<A> acc = RunSum<A>::of(Op<A>::zero());
     bool spread = false;  // acc is nonzero in lanes other than lane 0
 
-    for (;;) {  // blocks of empty segments
+    while (w < nblk) {  // blocks of empty segments
         unsigned m = __ballot_sync(0xffffffffu, blk0 == blk1);
         for (; m != 0u; m &= m - 1u) {
             const int64_t b = __shfl_sync(0xffffffffu, blk, __ffs(m) - 1);
