@@ -129,9 +129,12 @@ typedef enum {
                                    ignored; deterministic.  Shape fields other than grid
                                    must be 0 or the form's nominal shape, which
                                    sr_plan_segmented reports (16-byte vectors, unroll 2,
-                                   256 threads; else SR_ERR_UNSUPPORTED); an explicit grid
-                                   of more than 4 CTAs per SM -> SR_ERR_LAUNCH.  Not with
-                                   another form flag.  The paper has no counterpart. */
+                                   256 threads; else SR_ERR_UNSUPPORTED) though CTAs of 384
+                                   threads with 32-byte vectors run; ctas_per_sm and stages
+                                   are ignored; the grid is an explicit one (more than 4
+                                   CTAs per SM -> SR_ERR_LAUNCH) or the CTAs the device
+                                   holds.  Not with another form flag.  The paper has no
+                                   counterpart. */
 #define SR_F_HOST_DIRECT 0x800  /* sr_reduce_sum_host only: the kernel reads the host
                                    array in place over the CPU-GPU link (page-locked
                                    memory, or any memory where the device accesses
@@ -235,6 +238,8 @@ int sr_reduce_sum(const void* x, int64_t n, int dtype, void* out, int variant,
  * SR_AUTO / SR_TWO_KERNEL with optional SR_F_KAHAN / SR_F_FP64_COMBINE and
  * launch-shape fields; other stages or SR_F_BULK -> SR_ERR_UNSUPPORTED.
  * The first call that copies allocates the stream's staging buffers (128 MiB).
+ * Threads may share a stream: copying calls then take turns, and at most 64
+ * calls have their result under way at a time.
  * With SR_F_HOST_DIRECT there is no staging: one reduction (LDG path, stage
  * SR_LAST_BLOCK) reads x through its device mapping; SR_ERR_UNSUPPORTED when x
  * is neither page-locked nor accessible as pageable memory on this device.
@@ -297,7 +302,7 @@ int sr_plan(int64_t n, int dtype, const sr_config* cfg, sr_config* resolved);
  * explicit shape (vec_bytes, unroll, block_threads and stages all 0) calls
  * with 32768 or more segments take the TMA form, fewer the LDG one — or, from
  * 4096 segments, with no stage, grid or ctas_per_sm asked for either, the form of
- * SR_F_ADAPTIVE_SEGMENTS.
+ * SR_F_ADAPTIVE_SEGMENTS (SR_I32 with the atomic finish).
  * With SR_F_WARP_SEGMENTS whole segments go to single warps instead, with
  * SR_F_LANE_SEGMENTS to single threads (see the flags): no segment is split,
  * the stage bits are ignored and the results are deterministic.  With
@@ -534,8 +539,8 @@ int sr_reduce_sum_selected(sr_selector selector, const void* x, int64_t n, int d
  * can route a layout with a very long segment to the lane or warp form, where
  * one thread or one warp sums that segment alone (still correct, but up to
  * hundreds of times slower than the plain form).  Callers without reliable
- * statistics should use SR_F_ADAPTIVE_SEGMENTS, whose speed does not depend on
- * how the lengths are distributed.
+ * statistics should use SR_F_ADAPTIVE_SEGMENTS, which needs none: it splits by
+ * elements and shares long runs of empty segments among its warps.
  * Returns the flag, or a negated status: -SR_ERR_DTYPE, -SR_ERR_ARG (sms < 1,
  * nseg < 0, negative or NaN statistics). */
 int sr_segmented_layout_flags(int sms, int dtype, int64_t nseg, double len_mean, double len_std, double len_max);

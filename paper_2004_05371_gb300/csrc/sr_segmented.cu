@@ -163,10 +163,11 @@ int seg_plan(int64_t nseg, int dtype, const sr_config& c, const DeviceInfo& d, S
     // With nothing asked for, kSegAdaptMin or more segments (below kSegBulkMin)
     // take the adaptive form: the LDG kernel pays for every segment end with a
     // masked row and a warp reduction (20,000 lognormal segments of 2000 BF16
-    // values 48.6 us against 21.2; 14,454 of 445 f32 24.4 against 11.9; 10,000 of
-    // 26,844 f32 159 against 158).  With fewer, each segment spans many warps and the
-    // LDG kernel's shorter start wins (1000 of 1000 int32 5.7 us against 10.0; 2000
-    // of 400 f32 8.5 against 9.7; 3000 of 50 f32 8.8 against 8.5).
+    // values 43.4 us against 22.3; 14,454 of 445 f32 20.2 against 11.3; 10,000 of
+    // 26,844 f32 161 against 160; small ones: 4096 of 256 f32 9.1 against 8.9, of 16 8.9
+    // against 8.8, 6000 of 64 9.4 against 8.8; the worst of 300 sizes, 4096 of 547 BF16,
+    // 9.2 against 10.0).  With fewer, each segment spans many warps and the LDG
+    // kernel's shorter start wins (1000 of 1000 int32 6.7 us against 10.1).
     const bool shape_given = c.vec_bytes || c.unroll || c.block_threads || c.stages;
     p.adapt = (c.variant & SR_F_ADAPTIVE_SEGMENTS) != 0 ||
               (!shape_given && !c.grid && !c.ctas_per_sm && nseg >= kSegAdaptMin && nseg < kSegBulkMin &&
@@ -176,9 +177,10 @@ int seg_plan(int64_t nseg, int dtype, const sr_config& c, const DeviceInfo& d, S
         // (deterministic).  It balances the warps by elements whatever the
         // lengths, and resolves short and long segments alike; against the
         // device-side partition into lanes, lane groups and queued chunks it
-        // replaced (~2^28 elements): 4M lognormal f32 366 -> 200 us, 10,000
-        // lognormal 196 -> 162, 16M x 16 246 -> 229; 4M x 39 lognormal bf16 154
-        // -> 115.  The form's nominal shape is all a caller may name.
+        // replaced (~2^28 elements): 4M lognormal f32 366 -> 190 us, 10,000
+        // lognormal 196 -> 160, 16M x 16 246 -> 214; 4M x 39 lognormal bf16 154
+        // -> 108; 4M empty segments 39 -> 7.  The form's nominal shape is all a
+        // caller may name.
         if ((c.vec_bytes && c.vec_bytes != 16) || (c.unroll && c.unroll != 2) ||
             (c.block_threads && c.block_threads != 256))
             return SR_ERR_UNSUPPORTED;

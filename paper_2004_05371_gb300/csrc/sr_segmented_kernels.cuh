@@ -110,8 +110,6 @@ __device__ __forceinline__ int64_t warp_search(const int64_t* off, int64_t nseg,
     return lo + __ffs(__ballot_sync(0xffffffffu, lo + lane >= hi || win >= key)) - 1;
 }
 
-// Element j of a vector held as 32-bit words (the masked slow path; j is a
-// compile-time constant after unrolling).
 // Bits j of a PV-bit mask with a <= j < b (a and b clamped to [0, PV]).
 template <int PV> __device__ __forceinline__ uint32_t run_mask(int64_t a, int64_t b) {
     const int ja = a <= 0 ? 0 : (a >= PV ? PV : (int)a);
@@ -134,6 +132,8 @@ template <class A, int W> __device__ __forceinline__ A sum_words(const A (&acc)[
     return t[0];
 }
 
+// Element j of a vector held as 32-bit words (the masked slow path; j is a
+// compile-time constant after unrolling).
 template <int DT, class A> __device__ __forceinline__ void acc_vec_elem(A& a, const uint32_t* r, int j);
 template <> __device__ __forceinline__ void acc_vec_elem<kDtI32, long long>(long long& a, const uint32_t* r, int j) {
     a += (long long)(int)r[j];
@@ -573,13 +573,14 @@ __global__ void __launch_bounds__(512, 1) seg_kernel(const SegParams p) {
 //
 // Resolving the ends row by row, with a warp reduction for each (as the LDG
 // kernel does), bounded the ring by its instructions: it read 1M segments of 268
-// BF16 values at 1.8 TB/s.  Now a chunk with ends in it costs about 450 warp
-// instructions whatever their number, where HBM leaves time for some 650.
+// BF16 values at 1.8 TB/s.  Now a chunk without an end costs 160 warp instructions, one
+// with a few 460 to 510 (f32 4M x 64, bf16 1M x 268), one with 64 690 (i32 2M x 16), and
+// an FP8 one with 100 2100; HBM leaves time for some 650.
 // Device time before and now (~2^28 elements unless said otherwise):
-//   f32   1M x 268             343 -> 177 us      f32  4M lognormal    1013 -> 191 us
-//   f32   4M x 64              915 -> 188         f32  16M x 16        3110 -> 209
-//   bf16  1M x 268 (0..536)    297 -> 100         fp8  100k lognormal   160 ->  61
-//   i32   2^21 x 16 (0..32)    525 ->  53         bf16 4M x 39, lognormal 868 -> 113
+//   f32   1M x 268             343 -> 179 us      f32  4M lognormal    1013 -> 190 us
+//   f32   4M x 64              915 -> 191         f32  16M x 16        3110 -> 214
+//   bf16  1M x 268 (0..536)    297 -> 100         fp8  100k lognormal   160 ->  60
+//   i32   2^21 x 16 (0..32)    525 ->  53         bf16 4M x 39, lognormal 870 -> 108
 // What bounds it now: instructions (55-70 % of the issue slots) from about five
 // ends per chunk up, HBM below, and 4-7 us of search and first copies at the start.
 // 80 registers, so 24 warps (two 384-thread CTAs, 1 % ahead of three of 256) are

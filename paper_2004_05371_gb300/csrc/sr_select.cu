@@ -267,7 +267,7 @@ int sr_reduce_sum_segmented_selected(sr_selector s, const void* x, const int64_t
 //    short segments summed by single lanes), thread 991, LDG rows 973;
 //  - 10^4-10^5 lognormal segments: the flat split; the whole-segment forms are
 //    13-500x slower there, one warp or thread holding a segment of millions.
-// The strip kernel, without statistics, takes 210, 189, 177 and 192 us on the
+// The strip kernel, without statistics, takes 215, 191, 179 and 189 us on the
 // first four: ahead of the warp form, which this rule still names.
 // The dense kernel (a warp-wide pass over rows with many segment ends) is
 // 1.4-5.5x the plain kernel on uniformly short segments of fewer segments.
